@@ -480,7 +480,7 @@ __device__ __forceinline__ float binary_area(const float4* nodes, int c) {
 constexpr int EMPTY4 = (int)0x80000000;
 
 __global__ void k_collapse(const float4* nodes, const int* qin, int nin, int* qout, int* counters, int* src4,
-                           float4* nodes4) {
+                           float4* nodes4, int* parent4, int* leaf_node4) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nin) return;
   int b = qin[2 * k], id = qin[2 * k + 1];
@@ -510,6 +510,9 @@ __global__ void k_collapse(const float4* nodes, const int* qin, int nin, int* qo
       qout[2 * qi] = sj;
       qout[2 * qi + 1] = nid;
       child[j] = nid;
+      parent4[nid] = id;
+    } else if (sj != EMPTY4) {
+      leaf_node4[~sj] = id;
     }
     src4[4 * id + j] = sj;
   }
@@ -567,12 +570,14 @@ cudaError_t bvh_collapse(st_scene* s, cudaStream_t stream) {
   int* qb = s->q4 + 2 * (size_t)n;
   cudaError_t e = cudaMemcpyAsync(qa, init, sizeof(init), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(s->c4, cnt, sizeof(cnt), cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->parent4, 0xff, sizeof(int), stream);   // the root has no parent
   int nin = 1;
   for (int level = 0; nin > 0 && e == cudaSuccess; ++level) {
     if (level > 64) return cudaErrorIllegalState;  // deeper than any tree built here: malformed
     e = cudaMemsetAsync(s->c4 + 1, 0, sizeof(int), stream);
     if (e != cudaSuccess) break;
-    k_collapse<<<(nin + 127) / 128, 128, 0, stream>>>(s->nodes, qa, nin, qb, s->c4, s->src4, s->nodes4);
+    k_collapse<<<(nin + 127) / 128, 128, 0, stream>>>(s->nodes, qa, nin, qb, s->c4, s->src4, s->nodes4,
+                                                    s->parent4, s->leaf_node4);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, s->c4, sizeof(cnt), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -590,6 +595,7 @@ int sort_blocks_for(int n) { return (n + RS_TILE - 1) / RS_TILE; }
 __global__ void k_mesh_stat_init(MeshStat* m) {
   m->vol6 = 0.0;
   m->winding = 0;
+  m->lmax2 = 0;
   for (int k = 0; k < 3; ++k) {
     m->lo[k] = 0x7fffffff;
     m->hi[k] = (int)0x80000000;
@@ -599,16 +605,26 @@ __global__ void k_mesh_stat_init(MeshStat* m) {
 __global__ void k_mesh_stat(const float* V, int nv, const int* F, int nf, MeshStat* m) {
   __shared__ double sv[8];
   double v = 0.0;
+  float l2 = 0.0f;
   for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
     const int* fi = F + 3 * f;
+    float3 p0 = mk3(V[3 * fi[0]], V[3 * fi[0] + 1], V[3 * fi[0] + 2]), p1 = mk3(V[3 * fi[1]], V[3 * fi[1] + 1], V[3 * fi[1] + 2]),
+           p2 = mk3(V[3 * fi[2]], V[3 * fi[2] + 1], V[3 * fi[2] + 2]);
+    l2 = fmaxf(l2, fmaxf(dot3(p1 - p0, p1 - p0), fmaxf(dot3(p2 - p0, p2 - p0), dot3(p2 - p1, p2 - p1))));
     double a[3], b[3], c[3];
     for (int k = 0; k < 3; ++k) {
       a[k] = V[3 * fi[0] + k]; b[k] = V[3 * fi[1] + k]; c[k] = V[3 * fi[2] + k];
     }
     v += a[0] * (b[1] * c[2] - b[2] * c[1]) - a[1] * (b[0] * c[2] - b[2] * c[0]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
   }
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = v;
+  for (int o = 16; o > 0; o >>= 1) {
+    v += __shfl_xor_sync(0xffffffffu, v, o);
+    l2 = fmaxf(l2, __shfl_xor_sync(0xffffffffu, l2, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sv[threadIdx.x >> 5] = v;
+    atomicMax(&m->lmax2, __float_as_int(l2));
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
@@ -639,6 +655,7 @@ __global__ void k_mesh_stat_final(MeshStat* m) {
   double d[3];
   for (int k = 0; k < 3; ++k) d[k] = (double)unordered(m->hi[k]) - (double)unordered(m->lo[k]);
   double box6 = 6.0 * d[0] * d[1] * d[2];
+  m->eta = 1e-6f * sqrtf(__int_as_float(m->lmax2));
   m->winding = fabs(m->vol6) > 1e-3 * box6 ? (m->vol6 > 0.0 ? 1 : -1) : 0;
 }
 

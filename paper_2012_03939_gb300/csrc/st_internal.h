@@ -13,11 +13,13 @@ namespace st {
 
 // Mesh facts the primary-visibility bins use to drop back faces: six times the
 // signed volume (its sign tells outward from inward winding) and the vertex
-// bounds as order-preserving ints.
+// bounds as order-preserving ints; and for the horizons the longest edge.
 struct MeshStat {
   double vol6;
   int lo[3], hi[3];
   int winding;   // +1 outward, -1 inward, 0 when the volume is too small against the bounds to tell
+  int lmax2;     // longest edge, squared (float bits)
+  float eta;     // 1e-6 of the longest edge: how far beside a triangle the watertight test may report a hit
 };
 
 // Per-call arguments the kernels read from device memory, so a captured CUDA
@@ -176,6 +178,14 @@ struct st_scene {
   int lbin_res = 0;
   bool lbins_valid = false;
   unsigned long long lbins_geom = 0;
+  int* parent4 = nullptr;        // [n4] parent of each 4-wide node (-1: root), [F] node of each leaf: leaf_node4
+  int* leaf_node4 = nullptr;
+  // the faces' free directions (st_horizon.cuh), those of the vertices of geom_version == hz_geom
+  uint4* hz = nullptr;           // [F] marked cells per leaf
+  float4* hz_nodes = nullptr;    // [3 * n4] node records they are built through
+  int* hz_done = nullptr;        // [n4] their bottom-up counters
+  bool hz_valid = false;
+  unsigned long long hz_geom = 0;
   float* acc = nullptr;          // [6 * pixels] forward accumulation, compensated FP32 (sum, error) per channel
   unsigned long long* sacc = nullptr;  // [pixels] path-signature sums (bin-space pixel index)
   long long acc_cap = 0;
@@ -199,7 +209,7 @@ struct st_scene {
   int ev_used[3] = {0, 0, 0};
   int host_syncs = 0;
   int sm_count = 0;
-  int g_ext = 0, g_ext_s = 0, g_shade = 0, g_shadow = 0, g_shadow_s = 0;  // stage grids
+  int g_ext = 0, g_ext_s = 0, g_shade = 0, g_shade_hz = 0, g_shadow = 0, g_shadow_s = 0;  // stage grids
   long long last_edge_samples = 0;
   int launches = 0;              // kernels enqueued by the last call
   st_stats last{};

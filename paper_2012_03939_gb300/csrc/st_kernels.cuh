@@ -10,6 +10,7 @@
 // counter, so the same launch works for any queue length (needed for CUDA
 // graph replay, where the host never reads the counts).
 #pragma once
+#include "st_horizon.cuh"
 #include "st_internal.h"
 #include "st_trace.cuh"
 
@@ -59,6 +60,7 @@ struct KCtx {
   const int* lbin_ok;     // per scene light: 1 = its shadow rays may use the lists
   long long lbin_cap;
   long long lbin_cells;
+  const uint4* hz;        // per leaf, the face's marked cells (st_horizon.cuh); nullptr: every ray is traced
   float* acc;             // per-pixel compensated sample sums, (sum, error) x 3 (bin-space pixel index)
   int cull;               // the mesh is one closed, consistently wound surface (see MeshStat)
   const MeshStat* mstat;
@@ -905,6 +907,7 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_extend(KCtx c, int b, int fb) {
     float4 o = E.o[slot], d = E.d[slot];
     float t = __int_as_float(0x7f800000);
     int fl = -1;
+    if (!(d.w < 0.0f))   // else known to leave the mesh (k_shade)
     trace_bvh<false, STATS>(c.nodes, c.tri, c.nf, c.n4, xyz(o), xyz(d), __int_as_float(0x7f800000), E.origin[slot], t,
                             sstack + threadIdx.x, c.err, &ts, &fl);
     E.hit[slot] = make_int2(fl, __float_as_int(t));   // leaf index: shading reads the contiguous leaf record
@@ -923,12 +926,35 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_extend(KCtx c, int b, int fb) {
   }
 }
 
+// Environment radiance seen by an escaping ray, times the weight of a BSDF sample of pdf lp (b > 0) against the
+// environment's own sampling; tx = the texel it reads.
+__device__ __forceinline__ float3 escape_radiance(const KCtx& c, float3 dir, int b, float lp, int& tx) {
+  float st_;
+  tx = env_texel(c.env, dir, st_);
+  float4 te = __ldg(&c.env.tex[tx]);
+  float w = 1.0f;
+  if (b > 0) {
+    float pe = env_pdf(c.env, te.w, st_);
+    w = lp * lp / (lp * lp + pe * pe);
+  }
+  return mk3(te.x, te.y, te.z) * w;
+}
+
+// NEE rays of a vertex (sh_c.w): not sent, to trace, known to reach the light (above the face's horizon)
+constexpr float SH_NONE = 0.0f, SH_TRACE = 1.0f, SH_FREE = 2.0f;
+
+// A vertex whose NEE rays all leave above its face's horizon (st_horizon.cuh) adds them here, and a continuation
+// above it escapes here: such a path needs no queue, no ray state and no traversal. The sums take the same terms in
+// the same order as the queued way (k_shadow's lights, then the escape), rounded alike. HZ = false: no free directions
+// are built, every ray is traced (89 registers against 114).
+template <bool HZ>
 __global__ void k_shade(KCtx c, int b) {
   const Engine& E = c.e;
   const int* qin = (b & 1) ? E.q1 : E.q0;
   int* qout = (b & 1) ? E.q0 : E.q1;
   const size_t Q = (size_t)E.Q;
   Key key{c.args->k0, c.args->k1};
+  int n_free = 0, n_esc = 0;   // queries answered here: NEE rays, continuations
   ST_WARP_LOOP(E.cnt[CNT_EXT + b], &E.cnt[CNT_SHADE_FETCH + b])
   bool sh_any = false, cont = false;
   int slot = live_ ? qin[qi_] : 0;
@@ -944,17 +970,9 @@ __global__ void k_shade(KCtx c, int b) {
     if (h.x < 0) {
       if (c.sig) { sig_mix(hs, 0xffffffffu); E.sig[slot] = hs; }
       if (c.env.w > 0) {
-        float st_;
-        int tx = env_texel(c.env, dir, st_);
+        int tx;
+        float3 Lw = escape_radiance(c, dir, b, d4.w, tx);
         if (c.sig) { sig_mix(hs, (uint32_t)tx); E.sig[slot] = hs; }   // the nearest-texel lookup is a decision
-        float4 te = __ldg(&c.env.tex[tx]);
-        float w = 1.0f;
-        if (b > 0) {
-          float pe = env_pdf(c.env, te.w, st_);
-          float lp = d4.w;
-          w = lp * lp / (lp * lp + pe * pe);
-        }
-        float3 Lw = mk3(te.x, te.y, te.z) * w;
         float4 r = E.rad[slot];
         E.rad[slot] = make_float4(r.x + T.x * Lw.x, r.y + T.y * Lw.y, r.z + T.z * Lw.z, 0.0f);
         if (E.records && b > 0) E.esc[slot] = make_float4(Lw.x, Lw.y, Lw.z, 1.0f);
@@ -967,9 +985,12 @@ __global__ void k_shade(KCtx c, int b) {
       float3 v0 = xyz(ta), v1 = xyz(tb), v2 = xyz(tc);
       float3 ng = norm3(cross3(v1 - v0, v2 - v0));
       float3 wo = -dir;
-      float3 n = dot3(ng, wo) < 0.0f ? -ng : ng;
+      const bool back = dot3(ng, wo) < 0.0f;
+      float3 n = back ? -ng : ng;
       // shading normal: n, or interpolated; a direction counts only above both
-      float3 ns = c.smooth ? shading_normal(c, f, p, v0, v1, v2, dot3(ng, wo) < 0.0f ? -1.0f : 1.0f) : n;
+      float3 ns = c.smooth ? shading_normal(c, f, p, v0, v1, v2, back ? -1.0f : 1.0f) : n;
+      HzPoint hz;
+      if (HZ) hz = hz_point(c.mstat, c.hz, h.x, p, v0, v1, v2, n, !back);
       int tex = texel_of(c, f, p, v0, v1, v2);
       Mat m = fetch_mat(c.P, tex);
       if (c.sig) sig_mix(hs, (uint32_t)f);
@@ -978,38 +999,70 @@ __global__ void k_shade(KCtx c, int b) {
         E.r0[b * Q + slot] = make_float4(p.x, p.y, p.z, __int_as_float(f));
         E.nb[slot] = b + 1;
       }
+      // NEE rays: bit j = light j, bit 8 = the environment sample; sent (above the surface) and open (through free
+      // cells)
+      int sent = 0, open = 0;
       const int nlp = lights_of(c, vi);
+      auto lit = [&](float3 wi, float dist) {
+        return dot3(n, wi) > 0.0f && dist > 2.0f * T_EPS && (!c.smooth || dot3(ns, wi) > 0.0f);
+      };
+      if (HZ)
+        for (int j = 0; j < nlp; ++j) {
+          float4 lp, li;
+          point_light(c, vi, j, lp, li);
+          float3 dv = xyz(lp) - p;
+          float dist = len3(dv);
+          float3 wi = dv * (1.0f / dist);
+          if (lit(wi, dist)) {
+            sent |= 1 << j;
+            if (hz_free(hz, wi)) open |= 1 << j;
+          }
+        }
+      int etx = 0;
+      float esth = 0.0f;
+      float3 ewi = mk3(0, 0, 0), escale = mk3(0, 0, 0);
+      if (c.env.w > 0) {
+        U4 u = philox((uint32_t)ct.x, (uint32_t)ct.y, (uint32_t)(vb << 4) | 1u, (uint32_t)ct.z, key.k0, key.k1);
+        etx = env_pick(c.env, u.x, u.y);
+        if (c.sig) sig_mix(hs, (uint32_t)etx);
+        int row = etx / c.env.w, col = etx - row * c.env.w;
+        float uu = ((float)col + unif(u.z)) / (float)c.env.w, vq = ((float)row + unif(u.w)) / (float)c.env.h;
+        float cth, sph, cph;
+        sincosf(PI_F * vq, &esth, &cth);
+        sincosf(2.0f * PI_F * uu, &sph, &cph);
+        ewi = mk3(-esth * sph, cth, esth * cph);
+        if (esth > 0.0f && dot3(n, ewi) > 0.0f && (!c.smooth || dot3(ns, ewi) > 0.0f)) {
+          sent |= ENV_VIS;
+          if (HZ && hz_free(hz, ewi)) open |= ENV_VIS;
+        }
+      }
+      if (HZ) sh_any = (sent & ~open) != 0;
+      float3 L = mk3(0, 0, 0);          // the sum of the NEE rays when every one is free
       for (int j = 0; j < c.nlt; ++j) {
+        if (HZ && !sh_any && !(sent >> j & 1)) continue;
         float4 lp = make_float4(0, 0, 1, 0), li = make_float4(0, 0, 0, 0);
         if (j < nlp) point_light(c, vi, j, lp, li);
         float3 dv = xyz(lp) - p;
         float dist = len3(dv);
         float3 wi = dv * (1.0f / dist);
-        float ci = dot3(n, wi);
-        bool valid = j < nlp && ci > 0.0f && dist > 2.0f * T_EPS && (!c.smooth || dot3(ns, wi) > 0.0f);
+        const bool valid = HZ ? (sent >> j & 1) != 0 : j < nlp && lit(wi, dist);
         float3 cc = mk3(0, 0, 0);
         if (valid) cc = mul(mul(T, brdf_cos(c.brdf, c.fresnel, m, ns, wi, wo)), xyz(li)) * (1.0f / (dist * dist));
-        E.sh_dir[j * Q + slot] = make_float4(wi.x, wi.y, wi.z, dist - T_EPS);
-        E.sh_c[j * Q + slot] = make_float4(cc.x, cc.y, cc.z, valid ? 1.0f : 0.0f);
-        sh_any |= valid;
+        if (!HZ || sh_any) {
+          sh_any |= valid;
+          E.sh_dir[j * Q + slot] = make_float4(wi.x, wi.y, wi.z, dist - T_EPS);
+          E.sh_c[j * Q + slot] = make_float4(cc.x, cc.y, cc.z, !valid ? SH_NONE : (open >> j & 1) ? SH_FREE : SH_TRACE);
+        } else {
+          L = mk3(__fadd_rn(L.x, cc.x), __fadd_rn(L.y, cc.y), __fadd_rn(L.z, cc.z));
+        }
       }
       int flags = 0;
-      float3 ewi = mk3(0, 0, 0), escale = mk3(0, 0, 0);
       if (c.env.w > 0) {
-        U4 u = philox((uint32_t)ct.x, (uint32_t)ct.y, (uint32_t)(vb << 4) | 1u, (uint32_t)ct.z, key.k0, key.k1);
-        int tx = env_pick(c.env, u.x, u.y);
-        if (c.sig) sig_mix(hs, (uint32_t)tx);
-        int row = tx / c.env.w, col = tx - row * c.env.w;
-        float uu = ((float)col + unif(u.z)) / (float)c.env.w, vq = ((float)row + unif(u.w)) / (float)c.env.h;
-        float sth, cth, sph, cph;
-        sincosf(PI_F * vq, &sth, &cth);
-        sincosf(2.0f * PI_F * uu, &sph, &cph);
-        ewi = mk3(-sth * sph, cth, sth * cph);
-        bool valid = sth > 0.0f && dot3(n, ewi) > 0.0f && (!c.smooth || dot3(ns, ewi) > 0.0f);
+        const bool valid = (sent & ENV_VIS) != 0;
         float3 cc = mk3(0, 0, 0);
         if (valid) {
-          float4 te = __ldg(&c.env.tex[tx]);
-          float pe = env_pdf(c.env, te.w, sth);
+          float4 te = __ldg(&c.env.tex[etx]);
+          float pe = env_pdf(c.env, te.w, esth);
           float w = 1.0f;
           if (vb < c.B - 1) {
             float pb = brdf_pdf(c.brdf, m, ns, ewi, wo);
@@ -1019,30 +1072,66 @@ __global__ void k_shade(KCtx c, int b) {
           cc = mul(mul(T, brdf_cos(c.brdf, c.fresnel, m, ns, ewi, wo)), escale);
           flags |= ENV_VALID;
         }
-        E.sh_dir[c.nlt * Q + slot] = make_float4(ewi.x, ewi.y, ewi.z, __int_as_float(0x7f800000));
-        E.sh_c[c.nlt * Q + slot] = make_float4(cc.x, cc.y, cc.z, valid ? 1.0f : 0.0f);
-        sh_any |= valid;
+        if (!HZ || sh_any) {
+          sh_any |= valid;
+          E.sh_dir[c.nlt * Q + slot] = make_float4(ewi.x, ewi.y, ewi.z, __int_as_float(0x7f800000));
+          E.sh_c[c.nlt * Q + slot] = make_float4(cc.x, cc.y, cc.z, !valid ? SH_NONE : (open & ENV_VIS) ? SH_FREE : SH_TRACE);
+        } else {
+          L = mk3(__fadd_rn(L.x, cc.x), __fadd_rn(L.y, cc.y), __fadd_rn(L.z, cc.z));
+        }
       }
+      // all NEE rays are free: their sum is added now (k_shadow would add it)
+      const bool here = HZ && sent != 0 && !sh_any;
+      if (here) flags |= sent;
       if (E.records) {
         E.r2[b * Q + slot] = make_float4(ewi.x, ewi.y, ewi.z, __int_as_float(flags));
         E.r3[b * Q + slot] = make_float4(escale.x, escale.y, escale.z, __int_as_float(tex));
       }
-      E.o[slot] = make_float4(p.x, p.y, p.z, 0.0f);
-      E.origin[slot] = f;          // excluded by this vertex's shadow rays and by its continuation
+      bool esc = false;
+      float3 wi = mk3(0, 0, 0);
+      float pdf = 0.0f;
       if (vb < c.B - 1) {
         U4 u = philox((uint32_t)ct.x, (uint32_t)ct.y, (uint32_t)(vb << 4) | 2u, (uint32_t)ct.z, key.k0, key.k1);
-        float3 wi;
-        float pdf = brdf_sample(c.brdf, m, ns, wo, unif(u.x), unif(u.y), unif(u.z), wi);
+        pdf = brdf_sample(c.brdf, m, ns, wo, unif(u.x), unif(u.y), unif(u.z), wi);
         if (c.smooth && pdf > 0.0f && !(dot3(n, wi) > 0.0f)) pdf = 0.0f;   // below the face
         if (c.sig) sig_mix(hs, (unif(u.x) < lobe_prob(m) ? 1u : 0u) | (pdf > 0.0f ? 2u : 0u));
         if (pdf > 0.0f) {
           float3 Qv = brdf_cos(c.brdf, c.fresnel, m, ns, wi, wo);
           T = mul(T, Qv) * (1.0f / pdf);
-          E.thr[slot] = make_float4(T.x, T.y, T.z, 0.0f);
-          E.d[slot] = make_float4(wi.x, wi.y, wi.z, pdf);
           if (E.records) E.r1[(b + 1) * Q + slot] = make_float4(wi.x, wi.y, wi.z, pdf);
-          cont = true;
+          esc = HZ && hz_free(hz, wi);
+          // the escape is added after the NEE rays: here if they are done, else by the next bounce's launch,
+          // which the negated pdf tells that the ray hits nothing
+          cont = !esc || sh_any;
         }
+      }
+      if (here || (esc && !cont)) {
+        float4 r = E.rad[slot];
+        if (here) {
+          n_free += __popc(sent);
+          r = make_float4(__fadd_rn(r.x, L.x), __fadd_rn(r.y, L.y), __fadd_rn(r.z, L.z), 0.0f);
+          if (c.sig) sig_mix(hs, (uint32_t)sent);
+        }
+        if (esc && !cont) {
+          ++n_esc;
+          if (c.sig) sig_mix(hs, 0xffffffffu);
+          if (c.env.w > 0) {
+            int tx;
+            float3 Lw = escape_radiance(c, wi, 1, pdf, tx);
+            if (c.sig) sig_mix(hs, (uint32_t)tx);
+            r = make_float4(r.x + T.x * Lw.x, r.y + T.y * Lw.y, r.z + T.z * Lw.z, 0.0f);
+            if (E.records) E.esc[slot] = make_float4(Lw.x, Lw.y, Lw.z, 1.0f);
+          }
+        }
+        E.rad[slot] = r;
+      }
+      if (sh_any || cont) {
+        E.o[slot] = make_float4(p.x, p.y, p.z, 0.0f);
+        E.origin[slot] = f;          // excluded by this vertex's shadow rays and by its continuation
+      }
+      if (cont) {
+        E.thr[slot] = make_float4(T.x, T.y, T.z, 0.0f);
+        E.d[slot] = make_float4(wi.x, wi.y, wi.z, esc ? -pdf : pdf);
       }
       if (c.sig) E.sig[slot] = hs;
     }
@@ -1052,6 +1141,16 @@ __global__ void k_shade(KCtx c, int b) {
   int qn = warp_append(&E.cnt[CNT_EXT + b + 1], cont);
   if (cont) qout[qn] = slot;
   ST_WARP_LOOP_END
+  if (HZ) {
+    for (int off = 16; off > 0; off >>= 1) {
+      n_free += __shfl_xor_sync(FULL, n_free, off);
+      n_esc += __shfl_xor_sync(FULL, n_esc, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      if (n_free) atomicAdd(&E.stat[STAT_SHADOW], (unsigned long long)n_free);
+      if (n_esc) atomicAdd(&E.stat[STAT_EXT], (unsigned long long)n_esc);
+    }
+  }
 }
 
 template <bool STATS>
@@ -1070,10 +1169,15 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_shadow(KCtx c, int b) {
     int vis = 0;
     for (int k = 0; k < c.NS; ++k) {
       float4 sc = E.sh_c[k * Q + slot];
-      if (sc.w == 0.0f) continue;
+      if (sc.w == SH_NONE) continue;
+      ++traced;
+      if (sc.w == SH_FREE) {
+        L += xyz(sc);
+        vis |= (k < c.nlt) ? (1 << k) : ENV_VIS;
+        continue;
+      }
       float4 sd = E.sh_dir[k * Q + slot];
       float t;
-      ++traced;
       int2 lr = k < c.nl ? light_bin_range(c, k, p) : make_int2(-1, -1);
       int hf = lr.x >= 0 ? (bin_any_hit<STATS>(c, p, xyz(sd), sd.w, exclude, lr, &ts) ? 0 : -1)
                          : trace_bvh<true, STATS>(c.nodes, c.tri, c.nf, c.n4, p, xyz(sd), sd.w, exclude, t,
