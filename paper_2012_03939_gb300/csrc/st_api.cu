@@ -61,6 +61,9 @@ bool fault_now(int site) {
 namespace {
 
 constexpr int DEFAULT_CHUNK = 1 << 22;
+// Candidates per view whose screen records are kept (48 bytes each); the samples of later ones project their edge
+// themselves. A silhouette of the 1M-face mesh has some ten thousand edges.
+constexpr int EDGE_RECORDS = 1 << 15;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
 // A call uses the faces' free directions (k_horizon) from HZ_JOBS_PER_FACE paths per face on: a face costs 4 to 17 ns
@@ -248,6 +251,8 @@ DevView make_view(const st_view& v, int spp) {
   d.off = (uint32_t)v.pixel_offset;
   d.pix_off = v.pixel_offset;
   d.nvl = v.n_lights;
+  d.div_spp = make_div((uint32_t)spp);
+  d.div_w = make_div((uint32_t)v.width);
   for (int j = 0; j < 4; ++j) d.vl[j] = make_float4(0, 0, 0, 0);
   for (int j = 0; j < v.n_lights && j < ST_MAX_VIEW_LIGHTS; ++j) {
     d.vl[2 * j] = make_float4(v.lights[j].pos[0], v.lights[j].pos[1], v.lights[j].pos[2], 0.0f);
@@ -392,14 +397,18 @@ st_status ensure_tables(st_scene* s, int n_views, int n_segs, bool edges) {
     dfree(s->edge_cand);
     dfree(s->edge_ncand);
     size_t n = (size_t)n_views * std::max(s->n_edges, 1);
-    if (dalloc(&s->edge_flag, n) != cudaSuccess || dalloc(&s->edge_cand, n) != cudaSuccess ||
-        dalloc(&s->edge_ncand, (size_t)n_views) != cudaSuccess) {
+    s->edge_cap = std::min(s->n_edges, EDGE_RECORDS);
+    if (dalloc(&s->edge_flag, (size_t)n_views * edge_flag_ints(s->n_edges)) != cudaSuccess ||
+        dalloc(&s->edge_cand, n) != cudaSuccess || dalloc(&s->edge_ncand, (size_t)n_views) != cudaSuccess ||
+        dalloc(&s->edge_rec, 3 * (size_t)n_views * s->edge_cap) != cudaSuccess) {
+    dfree(s->edge_rec);
       dfree(s->edge_flag);
       dfree(s->edge_cand);
       dfree(s->edge_ncand);
       s->edge_cap_views = 0;
       cudaGetLastError();
       return fail(ST_ERR_OOM, "edge tables");
+      dfree(s->edge_rec);
     }
     s->edge_cap_views = n_views;
   }
@@ -508,6 +517,7 @@ KCtx make_ctx(st_scene* s, const Plan& p) {
   c.sh_cand = s->sh_cand; c.sh_ncand = s->sh_ncand;
   c.bin_start = p.bins ? s->bin_start : nullptr;   // nullptr: every primary ray traverses the BVH
   c.lviews = s->d_lviews;
+  c.edge_rec = s->edge_rec; c.edge_cap = s->edge_cap;
   c.lbin_start = p.lbins ? s->lbin_start : nullptr;   // nullptr: every shadow ray traverses the BVH
   c.lbin_list = s->lbin_list; c.lbin_ok = s->lbin_ok; c.lbin_cap = s->lbin_cap; c.lbin_cells = s->lbin_cells;
   c.hz = p.hz ? s->hz : nullptr;
@@ -803,18 +813,18 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
   }
   if (p.shadow && !p.pairs.empty()) {
     int np = (int)p.pairs.size();
-    dim3 g((s->n_edges + 255) / 256, (unsigned)np);
-    k_sh_flags<<<g, 256, 0, st>>>(c, s->d_pairs, np, s->sh_flag);
+    dim3 g(edge_tiles(s->n_edges), (unsigned)np);
+    k_sh_flags<<<g, EDGE_FLAG_BLOCK, 0, st>>>(c, s->d_pairs, s->sh_flag);
     KCtx cc = c;   // the ordered compaction of the primary candidates, on the shadow tables
     cc.edge_flag = s->sh_flag; cc.edge_cand = s->sh_cand; cc.edge_ncand = s->sh_ncand;
-    k_edge_compact<<<(unsigned)np, 1024, 0, st>>>(cc);
+    k_edge_compact<false><<<g, EDGE_TILE, 0, st>>>(cc);
     s->launches += 2;
   }
   if (p.edges) {
     Range r("edge candidates");
-    dim3 g((s->n_edges + 255) / 256, (unsigned)p.views.size());
-    k_edge_flags<<<g, 256, 0, st>>>(c, (int)p.views.size());
-    k_edge_compact<<<(unsigned)p.views.size(), 1024, 0, st>>>(c);
+    dim3 g(edge_tiles(s->n_edges), (unsigned)p.views.size());
+    k_edge_flags<<<g, EDGE_FLAG_BLOCK, 0, st>>>(c);
+    k_edge_compact<true><<<g, EDGE_TILE, 0, st>>>(c);
     s->launches += 2;
   }
   // Batched calls of several chunks rotate them over the engines, each on its own
@@ -999,7 +1009,7 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
     drop_graphs(s);
     dfree(s->sh_flag); dfree(s->sh_cand); dfree(s->sh_ncand); dfree(s->d_pairs);
     size_t n = p.pairs.size() * (size_t)std::max(s->n_edges, 1);
-    if (dalloc(&s->sh_flag, n) != cudaSuccess || dalloc(&s->sh_cand, n) != cudaSuccess ||
+    if (dalloc(&s->sh_flag, p.pairs.size() * edge_flag_ints(s->n_edges)) != cudaSuccess || dalloc(&s->sh_cand, n) != cudaSuccess ||
         dalloc(&s->sh_ncand, p.pairs.size()) != cudaSuccess || dalloc(&s->d_pairs, p.pairs.size()) != cudaSuccess) {
       dfree(s->sh_flag); dfree(s->sh_cand); dfree(s->sh_ncand); dfree(s->d_pairs);
       cudaGetLastError();
@@ -1145,7 +1155,7 @@ void destroy(st_scene* s) {
   dfree(s->flags); dfree(s->keys); dfree(s->keys2); dfree(s->ids); dfree(s->ids2); dfree(s->hist); dfree(s->bounds);
   dfree(s->nodes4); dfree(s->src4); dfree(s->q4); dfree(s->c4);
   dfree(s->lights); dfree(s->env_tex); dfree(s->env_alias); dfree(s->edge_v); dfree(s->edge_f);
-  dfree(s->edge_flag); dfree(s->edge_cand); dfree(s->edge_ncand);
+  dfree(s->edge_flag); dfree(s->edge_cand); dfree(s->edge_ncand); dfree(s->edge_rec);
   dfree(s->sh_flag); dfree(s->sh_cand); dfree(s->sh_ncand); dfree(s->d_pairs); dfree(s->d_views); dfree(s->d_segs);
   free_light_bins(s);
   if (s->lbin_total_host) cudaFreeHost(s->lbin_total_host);

@@ -73,8 +73,25 @@ struct DevView {
   long long bin_cell;      // first cell of the view in the primary-visibility bins
   int kb;                  // bin cells per pixel side (1, 2, 4 or 8)
   int nvl;                 // the view's own point lights (after the scene's)
+  uint2 div_spp, div_w;    // division of 32-bit job and pixel numbers by spp and W (div_by)
   float4 vl[4];            // (position, 0), (intensity, 0) per view light
 };
+
+// Division of a 32-bit number by an invariant divisor: Granlund and Montgomery, "Division by Invariant Integers using
+// Multiplication" (PLDI 1994), figure 4.1. (magic, l), l = ceil(log2 d).
+__host__ __forceinline__ uint2 make_div(uint32_t d) {
+  uint32_t l = 0;
+  while (l < 32 && (1ull << l) < d) ++l;
+  return make_uint2((uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1), l);
+}
+__device__ __forceinline__ uint32_t div_by(uint32_t n, uint2 d) {
+  uint32_t t = __umulhi(d.x, n);
+  return (t + ((n - t) >> min(d.y, 1u))) >> (d.y > 0u ? d.y - 1u : 0u);
+}
+// pixel of camera job `local` of a view
+__device__ __forceinline__ long long pixel_of(const DevView& v, long long local) {
+  return local >> 32 ? local / v.spp : (long long)div_by((uint32_t)local, v.div_spp);
+}
 
 __device__ __forceinline__ float3 cam_dir(const DevView& v, float px, float py) {
   float sx = 2.0f * px / (float)v.W - 1.0f;
