@@ -364,12 +364,15 @@ st_status grow_engine(st_scene* s, Engine& e, int Q, int B, int NS, bool records
   return ST_OK;
 }
 
-// The call's wavefront buffers: one engine, or all OVERLAP_ENGINES when consecutive
-// chunks are to overlap on their streams (see enqueue_body).
-st_status ensure_engine(st_scene* s, int Q, int B, int NS, bool records, bool sec, bool shadow, bool two) {
+// The call's wavefront buffers: one engine, or up to OVERLAP_ENGINES when consecutive chunks are to overlap on their
+// streams (see enqueue_body). Engines past OVERLAP_REQUIRED that do not fit are done without, in later calls too.
+st_status ensure_engine(st_scene* s, int Q, int B, int NS, bool records, bool sec, bool shadow, long long chunks) {
   st_status r = grow_engine(s, s->eng, Q, B, NS, records, sec, shadow);
-  for (int k = 0; r == ST_OK && two && k < OVERLAP_ENGINES - 1; ++k)
-    r = grow_engine(s, s->eng2[k], Q, B, NS, records, sec, shadow);
+  for (int k = 1; r == ST_OK && k < std::min<long long>(chunks, s->max_engines); ++k) {
+    st_status x = grow_engine(s, s->eng2[k - 1], Q, B, NS, records, sec, shadow);
+    if (x != ST_OK && k < OVERLAP_REQUIRED) r = x;
+    else if (x != ST_OK) s->max_engines = k;
+  }
   return r;
 }
 
@@ -726,14 +729,19 @@ long long chunk_count(const Plan& p, int Q) {
   return (p.total + Q - 1) / Q;
 }
 
-// Overlap consecutive chunks on the engines: batched calls of two chunks or more whose grids are not sized on the
-// host and whose kernels are not timed one by one, once the further engines and the events are in place.
-bool overlap_chunks(const st_scene* s, const Plan& p, int Q, bool host_sized, bool timing) {
+// Engines that a call's consecutive chunks rotate over: more than one for batched calls of two chunks or more whose
+// grids are not sized on the host and whose kernels are not timed one by one, once their buffers and events are in place.
+int overlap_engines(const st_scene* s, const Plan& p, int Q, bool host_sized, bool timing) {
   long long nc = chunk_count(p, Q);
-  if (host_sized || timing || nc < 2 || (long long)s->xev.size() < nc + 2 * OVERLAP_ENGINES) return false;
-  for (int k = 0; k < OVERLAP_ENGINES - 1; ++k)
-    if (!s->aux_stream[k] || s->eng2[k].Q < Q || s->eng2[k].records != s->eng.records) return false;
-  return true;
+  if (host_sized || timing || nc < 2 || (long long)s->xev.size() < nc + 2 * OVERLAP_ENGINES) return 1;
+  int n = 1;
+  while (n < std::min<long long>(nc, s->max_engines) && s->aux_stream[n - 1] && s->eng2[n - 1].Q >= Q &&
+         s->eng2[n - 1].NS >= s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0) &&
+         (p.kind == 0 || (s->eng2[n - 1].records && s->eng2[n - 1].B >= p.B)) &&
+         (!p.sec || s->eng2[n - 1].sec_cap >= (long long)s->eng2[n - 1].B * s->eng2[n - 1].Q) &&
+         (!p.shadow || s->eng2[n - 1].shadow))
+    ++n;
+  return n;
 }
 
 st_status enqueue_call(st_scene* s, const Plan& p, int Q, cudaStream_t st, bool host_sized, bool timing) {
@@ -831,12 +839,13 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
   // stream, so one chunk's last, sparsely filled bounces and launch tails overlap
   // the next chunks' full stages. The auxiliary streams fork after the set-up
   // above and join before the finishing kernels; forward chunks resolve in order.
-  const bool multi = overlap_chunks(s, p, Q, host_sized, timing);
+  const int engines = overlap_engines(s, p, Q, host_sized, timing);
+  const bool multi = engines > 1;
   KCtx cx[OVERLAP_ENGINES];
   cudaStream_t sx[OVERLAP_ENGINES];
   cx[0] = c;
   sx[0] = st;
-  for (int k = 1; k < OVERLAP_ENGINES; ++k) {
+  for (int k = 1; k < engines; ++k) {
     cx[k] = c;
     cx[k].e = s->eng2[k - 1];
     cx[k].e.records = c.e.records;
@@ -848,11 +857,11 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
     if (multi) {
       cudaEvent_t fork = s->xev[s->xev_used++];
       ST_CUDA(cudaEventRecord(fork, st));
-      for (int i = 1; i < OVERLAP_ENGINES; ++i) ST_CUDA(cudaStreamWaitEvent(sx[i], fork, 0));
+      for (int i = 1; i < engines; ++i) ST_CUDA(cudaStreamWaitEvent(sx[i], fork, 0));
     }
     for (long long j0 = a; j0 < b; j0 += Q, ++k) {
       int n = (int)std::min<long long>(Q, b - j0);
-      int e = multi ? k % OVERLAP_ENGINES : 0;
+      int e = k % engines;
       cudaEvent_t done = multi && p.kind == 0 ? s->xev[s->xev_used++] : nullptr;
       st_status r = run_chunk(s, p, cx[e], j0, n, sx[e], host_sized, timing, overlaps(p, 0, j0, j0 + n),
                               overlaps(p, 1, j0, j0 + n), prev, done);
@@ -860,7 +869,7 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
       prev = done;
     }
     if (multi) {
-      for (int i = 1; i < OVERLAP_ENGINES; ++i) {
+      for (int i = 1; i < engines; ++i) {
         cudaEvent_t join = s->xev[s->xev_used++];
         ST_CUDA(cudaEventRecord(join, sx[i]));
         ST_CUDA(cudaStreamWaitEvent(st, join, 0));
@@ -896,7 +905,8 @@ std::vector<long long> graph_key(const Plan& p, int Q, const st_scene* s) {
   std::vector<long long> k = {p.kind, p.B, (long long)p.views.size(), Q, p.o.edge_term, p.o.edge_mode, p.o.edge_spp,
                               p.interior, p.edges, p.o.count_visits, p.bins, p.bins_reused, p.lbins,
                               p.lbins_reused, s->lbin_cap,
-                              p.o.persist_blocks, s->bin_cap, p.max_vl, p.sig, p.sec_tree, p.hz, p.hz_reused};
+                              p.o.persist_blocks, s->bin_cap, p.max_vl, p.sig, p.sec_tree, p.hz, p.hz_reused,
+                              overlap_engines(s, p, Q, false, false)};
   for (auto& v : p.views) {
     k.push_back(v.W); k.push_back(v.H); k.push_back(v.spp); k.push_back(v.pix_off); k.push_back(v.nvl);
   }
@@ -1064,7 +1074,7 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
   int NS = s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0);
   bool timing_call = p.o.time_kernels != 0;
   bool want_two = p.o.mode == ST_MODE_BATCHED && !timing_call && chunk_count(p, Q) >= 2;
-  r = ensure_engine(s, Q, p.B, NS, p.kind == 1, p.sec, p.shadow, want_two);
+  r = ensure_engine(s, Q, p.B, NS, p.kind == 1, p.sec, p.shadow, want_two ? chunk_count(p, Q) : 1);
   if (r != ST_OK) return r;
   if (want_two) {
     // events for the fork, every chunk's resolve and the join, made before any capture
