@@ -399,19 +399,19 @@ st_status ensure_tables(st_scene* s, int n_views, int n_segs, bool edges) {
     dfree(s->edge_flag);
     dfree(s->edge_cand);
     dfree(s->edge_ncand);
+    dfree(s->edge_rec);
     size_t n = (size_t)n_views * std::max(s->n_edges, 1);
     s->edge_cap = std::min(s->n_edges, EDGE_RECORDS);
     if (dalloc(&s->edge_flag, (size_t)n_views * edge_flag_ints(s->n_edges)) != cudaSuccess ||
         dalloc(&s->edge_cand, n) != cudaSuccess || dalloc(&s->edge_ncand, (size_t)n_views) != cudaSuccess ||
         dalloc(&s->edge_rec, 3 * (size_t)n_views * s->edge_cap) != cudaSuccess) {
-    dfree(s->edge_rec);
       dfree(s->edge_flag);
       dfree(s->edge_cand);
       dfree(s->edge_ncand);
+      dfree(s->edge_rec);
       s->edge_cap_views = 0;
       cudaGetLastError();
       return fail(ST_ERR_OOM, "edge tables");
-      dfree(s->edge_rec);
     }
     s->edge_cap_views = n_views;
   }
@@ -517,10 +517,10 @@ KCtx make_ctx(st_scene* s, const Plan& p) {
   c.env = s->env; c.brdf = s->brdf; c.fresnel = s->fresnel; c.res = s->res; c.ntex = s->ntex; c.np = s->np;
   c.edge_v = s->edge_v; c.edge_f = s->edge_f; c.n_edges = s->n_edges; c.edge_mode = p.o.edge_mode;
   c.edge_flag = s->edge_flag; c.edge_cand = s->edge_cand; c.edge_ncand = s->edge_ncand;
+  c.edge_rec = s->edge_rec; c.edge_cap = s->edge_cap;
   c.sh_cand = s->sh_cand; c.sh_ncand = s->sh_ncand;
   c.bin_start = p.bins ? s->bin_start : nullptr;   // nullptr: every primary ray traverses the BVH
   c.lviews = s->d_lviews;
-  c.edge_rec = s->edge_rec; c.edge_cap = s->edge_cap;
   c.lbin_start = p.lbins ? s->lbin_start : nullptr;   // nullptr: every shadow ray traverses the BVH
   c.lbin_list = s->lbin_list; c.lbin_ok = s->lbin_ok; c.lbin_cap = s->lbin_cap; c.lbin_cells = s->lbin_cells;
   c.hz = p.hz ? s->hz : nullptr;
@@ -577,8 +577,8 @@ st_status run_chunk(st_scene* s, const Plan& p, const KCtx& c, long long j0, int
   if (!s->g_ext) {
     s->g_ext = grid_of((const void*)k_extend<false>, EXT_BLOCK, sm);
     s->g_ext_s = grid_of((const void*)k_extend<true>, EXT_BLOCK, sm);
-    s->g_shade = grid_of((const void*)k_shade<false>, 256, sm);
-    s->g_shade_hz = grid_of((const void*)k_shade<true>, 256, sm);
+    s->g_shade = grid_of((const void*)k_shade<false>, SHADE_BLOCK, sm);
+    s->g_shade_hz = grid_of((const void*)k_shade<true>, SHADE_BLOCK, sm);
     s->g_shadow = grid_of((const void*)k_shadow<false>, EXT_BLOCK, sm);
     s->g_shadow_s = grid_of((const void*)k_shadow<true>, EXT_BLOCK, sm);
   }
@@ -622,7 +622,7 @@ st_status run_chunk(st_scene* s, const Plan& p, const KCtx& c, long long j0, int
         int qe = fb ? hc[CNT_FB] : q;
         launch = qe > 0;
         ge = std::max(1, (qe + EXT_BLOCK - 1) / EXT_BLOCK);
-        gs = (q + 255) / 256;
+        gs = (q + SHADE_BLOCK - 1) / SHADE_BLOCK;
       }
       Range rb(b == 0 ? "bounce 0" : b == 1 ? "bounce 1" : "bounce 2+");
       if (launch) {
@@ -632,8 +632,8 @@ st_status run_chunk(st_scene* s, const Plan& p, const KCtx& c, long long j0, int
         if (timing) ST_CUDA(cudaEventRecord(next_event(s, 0, false), st));
         s->launches++;
       }
-      if (k.hz) k_shade<true><<<gs, 256, 0, st>>>(k, b);
-      else k_shade<false><<<gs, 256, 0, st>>>(k, b);
+      if (k.hz) k_shade<true><<<gs, SHADE_BLOCK, 0, st>>>(k, b, fb ? 1 : 0);
+      else k_shade<false><<<gs, SHADE_BLOCK, 0, st>>>(k, b, fb ? 1 : 0);
       s->launches++;
       if (host_sized) {
         st_status r = read_counts();

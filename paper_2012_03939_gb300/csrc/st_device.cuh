@@ -287,6 +287,55 @@ __device__ __forceinline__ float3 brdf_cos(int brdf, int fr, const Mat& m, float
              m.kd[2] * kdc + (m.ks[2] + (1.0f - m.ks[2]) * x5) * spec);
 }
 
+// brdf_cos with every product and sum rounded as written. The compiler fuses a product into either side of a sum and
+// picks differently from kernel to kernel (with the register limit, too); shading's variants add the same terms and
+// have to agree bitwise.
+__device__ __forceinline__ float dot_rn(float3 a, float3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
+__device__ __forceinline__ float D_rn(int brdf, float c, float a) {
+  const float a2 = __fmul_rn(a, a), c2 = __fmul_rn(c, c);
+  if (brdf == 0) {
+    const float k = __fmaf_rn(c2, __fadd_rn(a2, -1.0f), 1.0f);
+    return a2 / __fmul_rn(__fmul_rn(PI_F, k), k);
+  }
+  const float tan2 = __fsub_rn(1.0f, c2) / c2;
+  return expf(-tan2 / a2) / __fmul_rn(__fmul_rn(__fmul_rn(PI_F, a2), c2), c2);
+}
+__device__ __forceinline__ float G1_rn(int brdf, float c, float a) {
+  if (brdf == 0) {
+    const float a2 = __fmul_rn(a, a);
+    const float q = sqrtf(__fmaf_rn(__fmul_rn(__fsub_rn(1.0f, a2), c), c, a2));
+    return __fmul_rn(2.0f, c) / __fadd_rn(c, q);
+  }
+  const float s2 = __fsub_rn(1.0f, __fmul_rn(c, c));
+  if (!(s2 > 0.0f)) return 1.0f;
+  const float x = c / __fmul_rn(a, sqrtf(s2));
+  const float e = expf(-__fmul_rn(x, x));
+  return 2.0f / __fadd_rn(__fadd_rn(1.0f, erff(x)), e / __fmul_rn(x, 1.7724538509055160f));
+}
+__device__ __forceinline__ float3 brdf_cos_rn(int brdf, int fr, const Mat& m, float3 n, float3 wi, float3 wo) {
+  const float ci = dot_rn(n, wi), co = dot_rn(n, wo);
+  if (!(ci > 0.0f) || !(co > 0.0f)) return mk3(0, 0, 0);
+  float3 h = mk3(__fadd_rn(wi.x, wo.x), __fadd_rn(wi.y, wo.y), __fadd_rn(wi.z, wo.z));
+  const float hl = sqrtf(dot_rn(h, h));
+  h = mk3(h.x / hl, h.y / hl, h.z / hl);
+  bool cl;
+  const float a = clamp_alpha(m.alpha, cl);
+  const float spec = __fmul_rn(__fmul_rn(D_rn(brdf, dot_rn(n, h), a), G1_rn(brdf, ci, a)), G1_rn(brdf, co, a)) /
+                     __fmul_rn(4.0f, co);
+  float x5 = 0.0f;
+  if (fr) {
+    const float x = __fsub_rn(1.0f, dot_rn(wi, h)), x2 = __fmul_rn(x, x);
+    x5 = __fmul_rn(__fmul_rn(x2, x2), x);
+  }
+  const float kdc = __fmul_rn(ci, 1.0f / PI_F);
+  auto ch = [&](int k) {
+    return __fmaf_rn(m.kd[k], kdc, __fmul_rn(__fmaf_rn(__fsub_rn(1.0f, m.ks[k]), x5, m.ks[k]), spec));
+  };
+  return mk3(ch(0), ch(1), ch(2));
+}
+
 // One-sample lobe-mixture pdf (solid angle) of direction wi.
 __device__ __forceinline__ float brdf_pdf(int brdf, const Mat& m, float3 n, float3 wi, float3 wo) {
   float ci = dot3(n, wi), co = dot3(n, wo);

@@ -147,12 +147,12 @@ struct st_scene {
   int* edge_flag = nullptr;      // [views * edge_flag_ints(E)]
   int* edge_cand = nullptr;      // [views * E]
   int* edge_ncand = nullptr;     // [views]
+  float4* edge_rec = nullptr;    // [views * edge_cap * 3] screen records of the candidates
+  int edge_cap = 0;
   int edge_cap_views = 0;
   int* sh_flag = nullptr;        // [pairs * edge_flag_ints(E)] light-silhouette flags per (view, light)
   int* sh_cand = nullptr;        // [pairs * E] their ordered compaction
   int* sh_ncand = nullptr;       // [pairs]
-  float4* edge_rec = nullptr;    // [views * edge_cap * 3] screen records of the candidates
-  int edge_cap = 0;
   int2* d_pairs = nullptr;       // [pairs] (view, light)
   int sh_cap_pairs = 0;
   // primary-visibility bins: per view pixel, the leaves whose screen box covers it

@@ -922,14 +922,17 @@ __global__ void k_raygen(KCtx c, long long j0, int n) {
       E.r1[i] = make_float4(d.x, d.y, d.z, 0.0f);
     }
     if (ok) {
+      // shading knows the rest of a first ray's state: its origin is the view's eye, its throughput 1
       if (c.sig) E.sig[i] = SIG_BASIS;
-      E.o[i] = make_float4(o.x, o.y, o.z, 0.0f);
       E.d[i] = make_float4(d.x, d.y, d.z, 0.0f);
-      E.thr[i] = make_float4(1, 1, 1, 0);
-      E.origin[i] = -1;
       E.ctr[i] = ct;
-      if (br.x >= 0) E.hit[i] = bin_closest<STATS>(c, o, d, br, tests);
-      else fb = true;
+      if (br.x >= 0) {
+        E.hit[i] = bin_closest<STATS>(c, o, d, br, tests);
+      } else {
+        E.o[i] = make_float4(o.x, o.y, o.z, 0.0f);
+        E.origin[i] = -1;
+        fb = true;
+      }
     }
   }
   int q = warp_append(&E.cnt[CNT_EXT + 0], ok);
@@ -947,19 +950,26 @@ __global__ void k_raygen(KCtx c, long long j0, int n) {
   }
 }
 
-// persistent fetch: a warp takes 32 consecutive queue entries per step
-#define ST_WARP_LOOP(total_expr, fetch_ptr)                                      \
-  const int lane_ = threadIdx.x & 31;                                          \
-  const int total_ = (total_expr);                                             \
-  for (;;) {                                                                   \
-    int base_ = 0;                                                             \
-    if (lane_ == 0) base_ = total_ > 0 ? atomicAdd((fetch_ptr), 32) : 0;       \
-    base_ = __shfl_sync(FULL, base_, 0);                                       \
-    if (base_ >= total_) break;                                                \
-    const int qi_ = base_ + lane_;                                             \
-    const bool live_ = qi_ < total_;
+// Persistent fetch: a warp takes up to 32 consecutive queue entries per step, the first ones by its own number (warps
+// of different blocks next to each other, so that a short queue spreads over all SMs), further ones from the counter.
+// A queue shorter than the grid's lanes is dealt out thinly, since its rays' lengths differ: a warp ends with its
+// longest ray, and lanes on different nodes take turns. Taking every entry from the counter cost an empty queue's
+// launch 23 us (5000 warps on one address, 4 us now), and 40k grazing rays in full warps of 3 active lanes 187 us.
+#define ST_WARP_LOOP(total_expr)                                                                   \
+  const int lane_ = threadIdx.x & 31;                                                              \
+  const int total_ = (total_expr);                                                                 \
+  const int warps_ = gridDim.x * (blockDim.x >> 5);                                                \
+  const int take_ = min(32, max(1, (total_ + warps_ - 1) / warps_));                               \
+  for (long long base_ = (long long)((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * take_; base_ < total_;) { \
+    const int qi_ = (int)base_ + lane_;                                                            \
+    const bool live_ = lane_ < take_ && qi_ < total_;
 
-#define ST_WARP_LOOP_END }
+#define ST_WARP_LOOP_END(fetch_ptr)                                     \
+    if ((long long)warps_ * take_ >= total_) break;                     \
+    int next_ = 0;                                                      \
+    if (lane_ == 0) next_ = atomicAdd((fetch_ptr), 32);                 \
+    base_ = (long long)warps_ * take_ + __shfl_sync(FULL, next_, 0);    \
+  }
 
 // Closest hits through the BVH: the rays of bounce b, or with fb = 1 the first
 // rays k_raygen queued because no bin cell serves them.
@@ -969,7 +979,7 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_extend(KCtx c, int b, int fb) {
   const Engine& E = c.e;
   const int* q = fb ? E.q1 : (b & 1) ? E.q1 : E.q0;
   TraceStats ts{0, 0};
-  ST_WARP_LOOP(fb ? E.cnt[CNT_FB] : E.cnt[CNT_EXT + b], fb ? &E.cnt[CNT_FB_FETCH] : &E.cnt[CNT_EXT_FETCH + b])
+  ST_WARP_LOOP(fb ? E.cnt[CNT_FB] : E.cnt[CNT_EXT + b])
   if (live_) {
     int slot = q[qi_];
     float4 o = E.o[slot], d = E.d[slot];
@@ -980,7 +990,7 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_extend(KCtx c, int b, int fb) {
                             sstack + threadIdx.x, c.err, &ts, &fl);
     E.hit[slot] = make_int2(fl, __float_as_int(t));   // leaf index: shading reads the contiguous leaf record
   }
-  ST_WARP_LOOP_END
+  ST_WARP_LOOP_END(fb ? &E.cnt[CNT_FB_FETCH] : &E.cnt[CNT_EXT_FETCH + b])
   if (!fb && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&E.stat[STAT_EXT], (unsigned long long)E.cnt[CNT_EXT + b]);
   if (STATS) {
     for (int off = 16; off > 0; off >>= 1) {
@@ -1003,7 +1013,7 @@ __device__ __forceinline__ float3 escape_radiance(const KCtx& c, float3 dir, int
   float w = 1.0f;
   if (b > 0) {
     float pe = env_pdf(c.env, te.w, st_);
-    w = lp * lp / (lp * lp + pe * pe);
+    w = __fmul_rn(lp, lp) / __fmaf_rn(pe, pe, __fmul_rn(lp, lp));
   }
   return mk3(te.x, te.y, te.z) * w;
 }
@@ -1014,16 +1024,20 @@ constexpr float SH_NONE = 0.0f, SH_TRACE = 1.0f, SH_FREE = 2.0f;
 // A vertex whose NEE rays all leave above its face's horizon (st_horizon.cuh) adds them here, and a continuation
 // above it escapes here: such a path needs no queue, no ray state and no traversal. The sums take the same terms in
 // the same order as the queued way (k_shadow's lights, then the escape), rounded alike. HZ = false: no free directions
-// are built, every ray is traced (89 registers against 114).
+// are built, every ray is traced (87 registers against 116).
+// Waits on loads with few warps (a third of the issue slots used at two blocks of 256 per SM), so it is held to seven
+// (without free directions six) blocks of 128: an iteration on 200k faces and 64 views 34.3 -> 31.9 ms, on 5120 faces
+// 3.91 -> 3.63, three planes 0.886 either way. What both variants add to a pixel is rounded as written (brdf_cos_rn).
+constexpr int SHADE_BLOCK = 128;
 template <bool HZ>
-__global__ void k_shade(KCtx c, int b) {
+__global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b, int first) {
   const Engine& E = c.e;
   const int* qin = (b & 1) ? E.q1 : E.q0;
   int* qout = (b & 1) ? E.q0 : E.q1;
   const size_t Q = (size_t)E.Q;
   Key key{c.args->k0, c.args->k1};
   int n_free = 0, n_esc = 0;   // queries answered here: NEE rays, continuations
-  ST_WARP_LOOP(E.cnt[CNT_EXT + b], &E.cnt[CNT_SHADE_FETCH + b])
+  ST_WARP_LOOP(E.cnt[CNT_EXT + b])
   bool sh_any = false, cont = false;
   int slot = live_ ? qin[qi_] : 0;
   if (live_) {
@@ -1031,9 +1045,10 @@ __global__ void k_shade(KCtx c, int b) {
     int4 ct = E.ctr[slot];
     const int vb = b + (ct.w & 15);   // path vertex this ray finds (side paths of edge samples start past 0)
     const int vi = ct.w >> 4;         // the path's view (its own lights)
-    float4 o4 = E.o[slot], d4 = E.d[slot];
+    const float3 org = first ? c.views[vi].eye : xyz(E.o[slot]);
+    float4 d4 = E.d[slot];
     float3 dir = xyz(d4);
-    float3 T = xyz(E.thr[slot]);
+    float3 T = first ? mk3(1, 1, 1) : xyz(E.thr[slot]);
     unsigned long long hs = c.sig ? E.sig[slot] : 0ull;
     if (h.x < 0) {
       if (c.sig) { sig_mix(hs, 0xffffffffu); E.sig[slot] = hs; }
@@ -1042,14 +1057,14 @@ __global__ void k_shade(KCtx c, int b) {
         float3 Lw = escape_radiance(c, dir, b, d4.w, tx);
         if (c.sig) { sig_mix(hs, (uint32_t)tx); E.sig[slot] = hs; }   // the nearest-texel lookup is a decision
         float4 r = E.rad[slot];
-        E.rad[slot] = make_float4(r.x + T.x * Lw.x, r.y + T.y * Lw.y, r.z + T.z * Lw.z, 0.0f);
+        E.rad[slot] = make_float4(__fmaf_rn(T.x, Lw.x, r.x), __fmaf_rn(T.y, Lw.y, r.y), __fmaf_rn(T.z, Lw.z, r.z), 0.0f);
         if (E.records && b > 0) E.esc[slot] = make_float4(Lw.x, Lw.y, Lw.z, 1.0f);
       }
     } else if (vb < c.B) {        // a ray past the last vertex adds nothing where it hits
       float4 ta = __ldg(&c.tri[3 * h.x]), tb = __ldg(&c.tri[3 * h.x + 1]), tc = __ldg(&c.tri[3 * h.x + 2]);
       int f = __float_as_int(ta.w);
       float t = __int_as_float(h.y);
-      float3 p = xyz(o4) + dir * t;
+      float3 p = mk3(__fmaf_rn(dir.x, t, org.x), __fmaf_rn(dir.y, t, org.y), __fmaf_rn(dir.z, t, org.z));
       float3 v0 = xyz(ta), v1 = xyz(tb), v2 = xyz(tc);
       float3 ng = norm3(cross3(v1 - v0, v2 - v0));
       float3 wo = -dir;
@@ -1079,7 +1094,7 @@ __global__ void k_shade(KCtx c, int b) {
           float4 lp, li;
           point_light(c, vi, j, lp, li);
           float3 dv = xyz(lp) - p;
-          float dist = len3(dv);
+          float dist = sqrtf(dot_rn(dv, dv));
           float3 wi = dv * (1.0f / dist);
           if (lit(wi, dist)) {
             sent |= 1 << j;
@@ -1111,11 +1126,11 @@ __global__ void k_shade(KCtx c, int b) {
         float4 lp = make_float4(0, 0, 1, 0), li = make_float4(0, 0, 0, 0);
         if (j < nlp) point_light(c, vi, j, lp, li);
         float3 dv = xyz(lp) - p;
-        float dist = len3(dv);
+        float dist = sqrtf(dot_rn(dv, dv));
         float3 wi = dv * (1.0f / dist);
         const bool valid = HZ ? (sent >> j & 1) != 0 : j < nlp && lit(wi, dist);
         float3 cc = mk3(0, 0, 0);
-        if (valid) cc = mul(mul(T, brdf_cos(c.brdf, c.fresnel, m, ns, wi, wo)), xyz(li)) * (1.0f / (dist * dist));
+        if (valid) cc = mul(mul(T, brdf_cos_rn(c.brdf, c.fresnel, m, ns, wi, wo)), xyz(li)) * (1.0f / (dist * dist));
         if (!HZ || sh_any) {
           sh_any |= valid;
           E.sh_dir[j * Q + slot] = make_float4(wi.x, wi.y, wi.z, dist - T_EPS);
@@ -1134,10 +1149,10 @@ __global__ void k_shade(KCtx c, int b) {
           float w = 1.0f;
           if (vb < c.B - 1) {
             float pb = brdf_pdf(c.brdf, m, ns, ewi, wo);
-            w = pe * pe / (pe * pe + pb * pb);
+            w = __fmul_rn(pe, pe) / __fmaf_rn(pb, pb, __fmul_rn(pe, pe));
           }
           escale = mk3(te.x, te.y, te.z) * (w / pe);
-          cc = mul(mul(T, brdf_cos(c.brdf, c.fresnel, m, ns, ewi, wo)), escale);
+          cc = mul(mul(T, brdf_cos_rn(c.brdf, c.fresnel, m, ns, ewi, wo)), escale);
           flags |= ENV_VALID;
         }
         if (!HZ || sh_any) {
@@ -1164,7 +1179,7 @@ __global__ void k_shade(KCtx c, int b) {
         if (c.smooth && pdf > 0.0f && !(dot3(n, wi) > 0.0f)) pdf = 0.0f;   // below the face
         if (c.sig) sig_mix(hs, (unif(u.x) < lobe_prob(m) ? 1u : 0u) | (pdf > 0.0f ? 2u : 0u));
         if (pdf > 0.0f) {
-          float3 Qv = brdf_cos(c.brdf, c.fresnel, m, ns, wi, wo);
+          float3 Qv = brdf_cos_rn(c.brdf, c.fresnel, m, ns, wi, wo);
           T = mul(T, Qv) * (1.0f / pdf);
           if (E.records) E.r1[(b + 1) * Q + slot] = make_float4(wi.x, wi.y, wi.z, pdf);
           esc = HZ && hz_free(hz, wi);
@@ -1187,7 +1202,7 @@ __global__ void k_shade(KCtx c, int b) {
             int tx;
             float3 Lw = escape_radiance(c, wi, 1, pdf, tx);
             if (c.sig) sig_mix(hs, (uint32_t)tx);
-            r = make_float4(r.x + T.x * Lw.x, r.y + T.y * Lw.y, r.z + T.z * Lw.z, 0.0f);
+            r = make_float4(__fmaf_rn(T.x, Lw.x, r.x), __fmaf_rn(T.y, Lw.y, r.y), __fmaf_rn(T.z, Lw.z, r.z), 0.0f);
             if (E.records) E.esc[slot] = make_float4(Lw.x, Lw.y, Lw.z, 1.0f);
           }
         }
@@ -1208,7 +1223,7 @@ __global__ void k_shade(KCtx c, int b) {
   if (sh_any) E.qs[qs] = slot;
   int qn = warp_append(&E.cnt[CNT_EXT + b + 1], cont);
   if (cont) qout[qn] = slot;
-  ST_WARP_LOOP_END
+  ST_WARP_LOOP_END(&E.cnt[CNT_SHADE_FETCH + b])
   if (HZ) {
     for (int off = 16; off > 0; off >>= 1) {
       n_free += __shfl_xor_sync(FULL, n_free, off);
@@ -1228,7 +1243,7 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_shadow(KCtx c, int b) {
   const size_t Q = (size_t)E.Q;
   int traced = 0;
   TraceStats ts{0, 0};
-  ST_WARP_LOOP(E.cnt[CNT_SH + b], &E.cnt[CNT_SH_FETCH + b])
+  ST_WARP_LOOP(E.cnt[CNT_SH + b])
   if (live_) {
     int slot = E.qs[qi_];
     float3 p = xyz(E.o[slot]);
@@ -1267,7 +1282,7 @@ __global__ void __launch_bounds__(EXT_BLOCK) k_shadow(KCtx c, int b) {
       E.r2[b * Q + slot] = make_float4(r2.x, r2.y, r2.z, __int_as_float(__float_as_int(r2.w) | vis));
     }
   }
-  ST_WARP_LOOP_END
+  ST_WARP_LOOP_END(&E.cnt[CNT_SH_FETCH + b])
   for (int off = 16; off > 0; off >>= 1) traced += __shfl_xor_sync(FULL, traced, off);
   if ((threadIdx.x & 31) == 0 && traced) atomicAdd(&E.stat[STAT_SHADOW], (unsigned long long)traced);
   if (STATS) {
