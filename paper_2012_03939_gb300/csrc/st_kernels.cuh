@@ -1415,7 +1415,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint(KCtx c, long long j0, int
   float3 A = mk3(0, 0, 0);
   if (esc) A = mul(g, xyz(E.esc[i]));
   float3 Pnext = mk3(0, 0, 0);
-  for (int b = c.B - 1; b >= 0; --b) {
+  // from the warp's deepest vertex: most paths of a convex mesh have one, and a warp of misses or edge sides none
+  for (int b = __reduce_max_sync(FULL, nbv) - 1; b >= 0; --b) {
     float vals[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) vals[k] = 0.0f;
