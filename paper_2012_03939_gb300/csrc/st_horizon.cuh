@@ -8,7 +8,7 @@
 // For a face f (unit normal n on the surface's outer side, MeshStat::winding;
 // in-plane axes T along the first edge and B = n x T) a cell is one of eight
 // 45-degree sectors of azimuth, each widened by HZ_WIDEN on both sides, times one
-// of 16 bands of the sine of elevation above HZ_FLOOR. A cell is marked when x - y
+// of 16 bands of the sine of elevation above HZ_FLOOR (hz_band). A cell is marked when x - y
 // may fall into it for some point x of another face and some y of f. Below
 // HZ_FLOOR nothing is free. The 128 bits are a uint4 per face. Sources of marks:
 //  - the nodes of the 4-wide tree, each with a centre, a radius, an axis (its
@@ -50,7 +50,10 @@
 // NEE and bounce rays answered: 99 % on the smooth spheres, 53 % on the knot, 80 % on
 // the rough mesh. Of an iteration on 200k faces and 64 views, k_extend and k_shadow
 // fell from 45.1 to 18.3 ms of kernel time, the iteration from 57.0 to 36.7 ms; one of
-// 1M rough faces and 8 views took 154 and takes 133 ms.
+// 1M rough faces and 8 views took 154 and takes 133 ms. (Those with the lowest band's
+// floor at 0.02; at 0.003, which answers grazing rays of gentle surfaces too, the
+// 200k-face iteration went from 31.4 to 30.0, one of 32 captures lit from the camera
+// from 5.76 to 5.29, both on the later kernels.)
 #pragma once
 #include "st_internal.h"
 #include "st_trace.cuh"
@@ -60,13 +63,18 @@ namespace st {
 constexpr float HZ_WIDEN = 0.1f;      // radians added to each side of a sector
 constexpr float HZ_RHO = 4.0f;        // largest rho for which the directions are used
 constexpr float HZ_MARGIN = 0.003f;   // constant part of the elevation margin (rounding of the frames)
-constexpr float HZ_FLOOR = 0.02f;     // sine of elevation below which nothing is free
-constexpr float HZ_BANDS = 16.0f / (1.0f - HZ_FLOOR);   // bands per unit of sine
+constexpr float HZ_FLOOR = 0.003f;    // sine of elevation below which nothing is free
+constexpr float HZ_LOW = 0.02f;       // upper end of the lowest band: what a gentle surface's neighbours reach
 constexpr int HZ_FEW = 1;             // cells not marked yet up to which a node is taken by its sphere too
 constexpr float HZ_FAR = 0.2f;        // radius over distance of a node (or triangle) taken by its sphere
 constexpr int HZ_WARPS = 8;           // warps (faces) of a k_horizon block
 constexpr int HZ_STACK = 96;          // nodes waiting to be opened; one past them marks its cells
 constexpr int HZ_OPEN = 512;          // nodes opened per face, likewise
+
+// position of a sine of elevation among the 16 bands: [HZ_FLOOR, HZ_LOW), then 15 of equal width up to 1
+__device__ __forceinline__ float hz_band(float s) {
+  return s < HZ_LOW ? (s - HZ_FLOOR) * (1.0f / (HZ_LOW - HZ_FLOOR)) : 1.0f + (s - HZ_LOW) * (15.0f / (1.0f - HZ_LOW));
+}
 
 // Normals of the sector borders (directions 45 k -+ HZ_WIDEN, k = 0..3) and the sector axes (22.5 + 45 k).
 struct HzLines {
@@ -268,7 +276,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
     struct Cells { unsigned w[4]; };
     auto cells = [&](unsigned sec, float lo, float hi) {
       Cells c;
-      int b0 = max(0, (int)floorf((lo - HZ_FLOOR) * HZ_BANDS - 1e-3f)), b1 = min(15, (int)floorf((hi - HZ_FLOOR) * HZ_BANDS + 1e-3f));
+      int b0 = max(0, (int)floorf(hz_band(lo) - 1e-3f)), b1 = min(15, (int)floorf(hz_band(hi) + 1e-3f));
       unsigned m = b1 >= b0 ? (2u << b1) - (1u << b0) : 0u;
 #pragma unroll
       for (int w = 0; w < 4; ++w) c.w[w] = (sec >> (2 * w) & 1u ? m : 0u) | (sec >> (2 * w + 1) & 1u ? m << 16 : 0u);
@@ -494,10 +502,10 @@ __device__ __forceinline__ HzPoint hz_point(const MeshStat* ms, const uint4* cel
 // True when a ray from the vertex along the unit direction d is known to hit nothing but its own face.
 __device__ __forceinline__ bool hz_free(const HzPoint& z, float3 d) {
   if (!z.on) return false;
-  float dn = dot3(d, z.n), lo = ((dn - z.lo) * z.irho - HZ_FLOOR) * HZ_BANDS;
+  float dn = dot3(d, z.n), lo = hz_band((dn - z.lo) * z.irho);
   if (!(lo >= 0.0f) || !(dn > z.least)) return false;
   int b0 = min((int)lo, 15), b1 = 15;
-  if (z.rho < 0.25f) b1 = min((int)(((dn + z.hi) * (1.0f + 1.34f * z.rho) - HZ_FLOOR) * HZ_BANDS), 15);   // / (1 - rho)
+  if (z.rho < 0.25f) b1 = min((int)hz_band((dn + z.hi) * (1.0f + 1.34f * z.rho)), 15);   // / (1 - rho)
   unsigned band = (2u << b1) - (1u << b0), w;
   if (z.rho * z.rho > HZ_WIDEN * HZ_WIDEN * (1.0f - dn * dn)) {   // the azimuth is too uncertain
     w = z.w.x | z.w.y | z.w.z | z.w.w;
