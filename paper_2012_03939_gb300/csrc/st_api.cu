@@ -772,6 +772,11 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
           s->et_lo, s->et_hi, s->et_cn, l);
     s->launches += 1 + s->et_L;
   }
+  // The faces' free directions are first needed by shading: built on their own stream beside the lists and candidates
+  // below, which leave most of the SMs' issue slots (calls timed kernel by kernel keep one stream). The build forks
+  // from here, and is enqueued after the set-up, so that a copy that fails there leaves nothing unjoined.
+  const bool hz_now = p.hz && !p.hz_reused, aside = hz_now && !host_sized && !timing;
+  if (aside) ST_CUDA(cudaEventRecord(s->hz_ev[0], st));
   if (p.bins && !p.bins_reused) {
     Range r("primary bins");
     // primary-visibility bins of every view: count, scan, fill
@@ -814,11 +819,6 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
     ST_CUDA(copy_async(s->lbin_total_host, s->lbin_start + P, sizeof(int), cudaMemcpyDeviceToHost, st));
     s->launches += 7;
   }
-  if (p.hz && !p.hz_reused) {
-    Range r("horizons");
-    ST_CUDA(hz_build(s, st));
-    s->launches += s->n4 > 0 ? 2 : 1;
-  }
   if (p.shadow && !p.pairs.empty()) {
     int np = (int)p.pairs.size();
     dim3 g(edge_tiles(s->n_edges), (unsigned)np);
@@ -834,6 +834,17 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
     k_edge_flags<<<g, EDGE_FLAG_BLOCK, 0, st>>>(c);
     k_edge_compact<true><<<g, EDGE_TILE, 0, st>>>(c);
     s->launches += 2;
+  }
+  if (hz_now) {
+    Range r("horizons");
+    if (aside) ST_CUDA(cudaStreamWaitEvent(s->hz_stream, s->hz_ev[0], 0));
+    cudaError_t e = hz_build(s, aside ? s->hz_stream : st);
+    if (aside) {
+      ST_CUDA(cudaEventRecord(s->hz_ev[1], s->hz_stream));
+      ST_CUDA(cudaStreamWaitEvent(st, s->hz_ev[1], 0));
+    }
+    ST_CUDA(e);
+    s->launches += s->n4 > 0 ? 2 : 1;
   }
   // Batched calls of several chunks rotate them over the engines, each on its own
   // stream, so one chunk's last, sparsely filled bounces and launch tails overlap
@@ -1181,6 +1192,9 @@ void destroy(st_scene* s) {
   if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
   for (auto a : s->aux_stream)
     if (a) cudaStreamDestroy(a);
+  if (s->hz_stream) cudaStreamDestroy(s->hz_stream);
+  for (auto v : s->hz_ev)
+    if (v) cudaEventDestroy(v);
   delete s;
 }
 
@@ -1365,6 +1379,8 @@ st_status st_scene_create(const st_scene_desc* d, void* stream, st_scene** out) 
   }
   chk(cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking));
   for (auto& a : s->aux_stream) chk(cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking));
+  chk(cudaStreamCreateWithFlags(&s->hz_stream, cudaStreamNonBlocking));
+  for (auto& v : s->hz_ev) chk(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
   if (e == cudaSuccess) e = s->builder == ST_BVH_LBVH ? bvh_build(s, st) : bvh_build_ploc(s, st);
   if (e == cudaSuccess) e = bvh_collapse(s, st);
   if (e == cudaSuccess) e = mesh_stat(s, st);

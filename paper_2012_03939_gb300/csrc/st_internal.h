@@ -190,6 +190,8 @@ struct st_scene {
   uint4* hz = nullptr;           // [F] marked cells per leaf
   float4* hz_nodes = nullptr;    // [3 * n4] node records they are built through
   int* hz_done = nullptr;        // [n4] their bottom-up counters
+  cudaStream_t hz_stream = nullptr;        // their build runs beside the call's other set-up
+  cudaEvent_t hz_ev[2] = {};               // its fork and join
   bool hz_valid = false;
   unsigned long long hz_geom = 0;
   float* acc = nullptr;          // [6 * pixels] forward accumulation, compensated FP32 (sum, error) per channel
