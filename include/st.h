@@ -236,7 +236,8 @@ st_status st_set_face_params(st_scene* scene, const float* face_params, void* st
  * graph on). Asynchronous on `stream`. Errors: ST_ERR_INVALID_ARG (bad views,
  * overlapping pixel ranges, no light), ST_ERR_UNSUPPORTED, ST_ERR_OOM, ST_ERR_CUDA;
  * a kernel's latched error is reported by st_get_stats (device_error).
- * A call of at least 2^20 primary rays finds their hits in screen-space leaf
+ * A call of at least 2^20 primary rays (5 * 2^17 for a closed mesh of few faces
+ * and views) finds their hits in screen-space leaf
  * lists of its views, kept on the device: a later call (forward or backward)
  * with the same views (camera, size) and no vertex update since uses them
  * without building them again. Such a call also bins the leaves, seen from each
