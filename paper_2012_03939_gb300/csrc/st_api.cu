@@ -292,6 +292,7 @@ struct Plan {
   bool sig = false;           // forward: path signatures
   int max_vl = 0;             // most point lights a view of the call adds to the scene's
   bool bins = false;          // build primary-visibility bins (worth it only for many primary rays)
+  bool cull = false;          // ... without the back faces of a closed mesh
   bool bins_reused = false;   // the previous build's lists serve this call (same views, same vertices)
   bool lbins = false;         // point-light shadow lists (scene lights, calls with many rays)
   bool lbins_reused = false;  // ... as the last build left them (no vertex update since)
@@ -484,10 +485,11 @@ st_status ensure_light_bins(st_scene* s) {
   return ST_OK;
 }
 
-// what the bins depend on besides the vertices: each view's camera frame, size and cell layout (bit patterns)
+// what the bins depend on besides the vertices: whether back faces are left out, and each view's camera frame, size and cell layout (bit patterns)
 std::vector<uint32_t> bins_key(const Plan& p) {
   std::vector<uint32_t> k;
   auto f = [&](float x) { uint32_t u; std::memcpy(&u, &x, 4); k.push_back(u); };
+  k.push_back(p.cull ? 1u : 0u);
   for (const DevView& v : p.views) {
     for (const float3& a : {v.eye, v.fwd, v.right, v.up}) { f(a.x); f(a.y); f(a.z); }
     f(v.kx); f(v.ky);
@@ -526,7 +528,7 @@ KCtx make_ctx(st_scene* s, const Plan& p) {
   c.hz = p.hz ? s->hz : nullptr;
   c.bin_list = s->bin_list; c.bin_cur = s->bin_cur; c.bin_ok = s->bin_ok;
   c.bin_cap = s->bin_cap; c.bin_pixels = p.pixels; c.bin_cells = p.cells;
-  c.cull = s->closed ? 1 : 0; c.mstat = s->mstat;
+  c.cull = p.cull ? 1 : 0; c.mstat = s->mstat;
   c.smooth = s->smooth ? 1 : 0; c.vn = s->vnrm; c.dN = s->dN; c.nv = s->nv;
   c.sec_tree = p.sec_tree ? 1 : 0; c.et_G = s->et_G; c.et_L = s->et_L; c.et_lo = s->et_lo; c.et_hi = s->et_hi;
   c.et_cn = s->et_cn;
@@ -914,7 +916,7 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
 
 std::vector<long long> graph_key(const Plan& p, int Q, const st_scene* s) {
   std::vector<long long> k = {p.kind, p.B, (long long)p.views.size(), Q, p.o.edge_term, p.o.edge_mode, p.o.edge_spp,
-                              p.interior, p.edges, p.o.count_visits, p.bins, p.bins_reused, p.lbins,
+                              p.interior, p.edges, p.o.count_visits, p.bins, p.cull, p.bins_reused, p.lbins,
                               p.lbins_reused, s->lbin_cap,
                               p.o.persist_blocks, s->bin_cap, p.max_vl, p.sig, p.sec_tree, p.hz, p.hz_reused,
                               overlap_engines(s, p, Q, false, false)};
@@ -1004,11 +1006,13 @@ st_status plan_call(st_scene* s, const st_view* views, int n_views, int default_
     return fail(ST_ERR_INVALID_ARG, "no light: the scene has none and no view brings one");
   // The lists cost a fixed 30 us (seven launches) and 0.14 ns per face and view to build. Below about a million primary
   // rays that exceeds what they save on an open mesh (three planes, 786k paths: 0.88 ms without, 0.93 with them); on a
-  // closed one, whose back faces they leave out, they pay from 5 * 2^17 on while there are few faces and views for the
-  // rays (1280 faces, 16 views, 801k paths, two calls on the same lists: 1.00 -> 0.70 ms).
+  // closed one they pay from 5 * 2^17 on while there are few faces and views for the rays (MATERIAL). Such calls keep
+  // the back faces in them: at a silhouette edge a ray can hit both faces within rounding, and the tree these calls
+  // used before takes the nearer of the two.
+  p.cull = s->closed && p.total >= (1LL << 20);
   p.bins = p.total >= (1LL << 20) ||
            (s->closed && p.total >= (5LL << 17) && (long long)s->nf * n_views <= p.total / 4);
-  p.lbins = p.bins && s->nl > 0;   // the same threshold: the build is a few launches over the faces
+  p.lbins = p.total >= (1LL << 20) && s->nl > 0;   // the same limit: the build is a few launches over the faces
   {
     std::vector<std::pair<long long, long long>> rg;
     for (int i = 0; i < n_views; ++i)

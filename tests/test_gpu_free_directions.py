@@ -116,3 +116,29 @@ def test_free_directions_skip_the_tree_on_a_convex_mesh(st):
     np.testing.assert_array_equal(img, fresh.render(sc.views, 3, 1).cpu().numpy())
     scene.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("mesh", ["sphere", "rough", "knot"])
+def test_lists_of_calls_below_a_million_rays_equal_the_tree(st, mesh):
+    """From 5 * 2^17 rays on a closed mesh's first rays are found in lists that keep its back faces: the same hits as
+    the tree's, at silhouettes too."""
+    V, F = _mesh(mesh, np.random.default_rng(8))
+    rng = np.random.default_rng(9)
+    views = S.fibonacci_views(4, [200, 129, 181, 97], [131, 177, 120, 210], [9, 9, 9, 8])
+    sc = S.Scene("lists", S._f32(V), np.ascontiguousarray(F, np.int32), S.random_face_params(rng, len(F)),
+                 env=S.lognormal_env(rng, 64, 32), views=views, max_bounces=2)
+    paths = sum(v.width * v.height * v.spp for v in views)
+    assert 5 << 17 <= paths < 1 << 20 and 4 * len(F) * len(views) <= paths
+    scene = st.Scene.from_scene(sc)
+    sig = torch.zeros(sc.n_pixels, dtype=torch.int64, device="cuda")
+    img = scene.render(views, 2, 11, st.make_opts(count_visits=1), signatures=sig)
+    many = scene.stats()
+    visits = 0
+    ref, s1 = torch.zeros_like(img), torch.zeros_like(sig)
+    for v in views:
+        scene.render([v], 2, 11, st.make_opts(count_visits=1), out=ref, signatures=s1)
+        visits += scene.stats()["node_visits"]
+    assert many["node_visits"] < 0.5 * visits   # the lists were used
+    np.testing.assert_array_equal(sig.cpu().numpy(), s1.cpu().numpy())
+    np.testing.assert_array_equal(img.cpu().numpy(), ref.cpu().numpy())
+    scene.close()
