@@ -545,34 +545,62 @@ __device__ __forceinline__ bool hidden_back_face(const KCtx& c, const DevView& v
   return w > 0 ? f < -tol : f > tol;
 }
 
-// fill = 0: count leaves per pixel; fill = 1: write them at start + cursor
+// fill = 0: count leaves per pixel; fill = 1: write them at start + cursor. A thread takes a leaf's cells when they are
+// few; a larger box is taken by the whole warp, a cell per lane: a coarse mesh seen at high resolution has hundreds of
+// cells per face, and their atomics one after the other held the launch up (1280 faces, two views of 66 x 433 pixels:
+// 0.60 ms to fill, now 0.03).
+constexpr int BIN_OWN_CELLS = 12;
 template <int FILL>
 __global__ void k_bin(KCtx c, int n_views, int* ok) {
-  int li = blockIdx.x * blockDim.x + threadIdx.x;
-  int vi = blockIdx.y;
-  if (li >= c.nf || vi >= n_views) return;
-  DevView v = c.views[vi];
+  const int li = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const int vi = blockIdx.y;
+  if (vi >= n_views) return;
+  const DevView v = c.views[vi];
   if (v.W <= 0) return;   // a light frustum that does not exist (k_light_views)
-  int x0, y0, x1, y1;
-  ScreenTri et;
-  float4 ta = __ldg(&c.tri[3 * li]), tb = __ldg(&c.tri[3 * li + 1]), tc = __ldg(&c.tri[3 * li + 2]);
-  if (hidden_back_face(c, v, ta, tb, tc)) return;
-  int r = leaf_screen_box(v, ta, tb, tc, x0, y0, x1, y1, et);
-  if (r < 0) { if (!FILL) atomicAnd(&ok[vi], 0); return; }
-  if (r == 0) return;
   if (FILL && c.bin_start[c.bin_cells] > c.bin_cap) return;   // overflow: every view uses the BVH
-  const long long Wc = (long long)v.W * v.kb;
-  for (int y = y0; y <= y1; ++y)
-    for (int x = x0; x <= x1; ++x) {
-      if (!pixel_may_overlap(et, x, y)) continue;
-      long long p = v.bin_cell + (long long)y * Wc + x;
-      int k = atomicAdd(&c.bin_cur[p], 1);
-      if (FILL) {
-        long long at = (long long)c.bin_start[p] + k;
-        if (at < c.bin_start[p + 1] && at < c.bin_cap) const_cast<int*>(c.bin_list)[at] = li;
-        else atomicOr(c.err, ERR_INDEX);
-      }
+  int x0 = 0, y0 = 0, x1 = -1, y1 = -1;
+  ScreenTri et;
+  et.degenerate = false;
+  if (li < c.nf) {
+    float4 ta = __ldg(&c.tri[3 * li]), tb = __ldg(&c.tri[3 * li + 1]), tc = __ldg(&c.tri[3 * li + 2]);
+    if (!hidden_back_face(c, v, ta, tb, tc)) {
+      int r = leaf_screen_box(v, ta, tb, tc, x0, y0, x1, y1, et);
+      if (r < 0 && !FILL) atomicAnd(&ok[vi], 0);
+      if (r <= 0) { x1 = x0 - 1; y1 = y0 - 1; }
     }
+  }
+  const long long Wc = (long long)v.W * v.kb;
+  auto put = [&](const ScreenTri& t, int leaf, int x, int y) {
+    if (!pixel_may_overlap(t, x, y)) return;
+    long long p = v.bin_cell + (long long)y * Wc + x;
+    int k = atomicAdd(&c.bin_cur[p], 1);
+    if (FILL) {
+      long long at = (long long)c.bin_start[p] + k;
+      if (at < c.bin_start[p + 1] && at < c.bin_cap) const_cast<int*>(c.bin_list)[at] = leaf;
+      else atomicOr(c.err, ERR_INDEX);
+    }
+  };
+  const int w = x1 - x0 + 1, n = w > 0 && y1 >= y0 ? w * (y1 - y0 + 1) : 0;   // at most BIN_MAX_BOX
+  if (n <= BIN_OWN_CELLS)
+    for (int y = y0; y <= y1; ++y)
+      for (int x = x0; x <= x1; ++x) put(et, li, x, y);
+  for (unsigned m = __ballot_sync(FULL, n > BIN_OWN_CELLS); m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    ScreenTri t;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      t.a[k] = __shfl_sync(FULL, et.a[k], src);
+      t.b[k] = __shfl_sync(FULL, et.b[k], src);
+      t.c[k] = __shfl_sync(FULL, et.c[k], src);
+    }
+    t.degenerate = __shfl_sync(FULL, et.degenerate ? 1 : 0, src) != 0;
+    const int leaf = __shfl_sync(FULL, li, src), bx = __shfl_sync(FULL, x0, src), by = __shfl_sync(FULL, y0, src),
+              bw = __shfl_sync(FULL, w, src), cells = __shfl_sync(FULL, n, src);
+    for (int i = lane; i < cells; i += 32) {
+      const int y = i / bw;
+      put(t, leaf, bx + (i - y * bw), by + y);
+    }
+  }
 }
 
 // ------------------------------------------------------------------ point-light shadow lists
