@@ -66,12 +66,16 @@ constexpr int DEFAULT_CHUNK = 1 << 22;
 constexpr int EDGE_RECORDS = 1 << 15;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
-// A call uses the faces' free directions (k_horizon) from HZ_JOBS_PER_FACE paths per face on: a face costs 4 to 17 ns
-// to build (smooth to rough; 1.6 ms at 200k faces, 16.8 ms at 1M), a path answered by them saves 0.1 to 0.3 ns. Below
-// HZ_MIN_JOBS paths the two launches' latency (50 us) is not won back; on an open mesh, whose faces mostly see one
-// another (three planes of 384 faces: a third of the cells empty, 0.97x at 786k paths), not below HZ_MIN_JOBS_OPEN.
+// Whether a call uses the faces' free directions (k_horizon). A face costs 8 (smooth) to 17 ns (rough) to build; of the
+// rays a path can send, those they spare the tree cost about 0.04 ns each (iterations on 5120 faces, B = 3, listed
+// lights only: 0.08 to 0.12 ns a path; 200k faces, B = 3, environment: 0.20; 1M rough ones, B = 5, environment: 0.32).
+// Those are the bounce rays and, where the call has other lights than the listed ones of the scene, the next-event rays;
+// a listed light's rays cost little without. An iteration's two calls share one build, so a call counts from HZ_GAIN
+// such rays per face on. Below HZ_MIN_JOBS paths the two launches' latency (50 us) is not won back; on an open mesh,
+// whose faces mostly see one another (three planes of 384 faces: a third of the cells empty, 0.97x at 786k paths), not
+// below HZ_MIN_JOBS_OPEN.
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
-constexpr int HZ_JOBS_PER_FACE = 16;
+constexpr int HZ_GAIN = 200;
 // Segment bases and chunk sizes are multiples of 64: an edge segment is laid out
 // in blocks of 64 jobs, the minus sides of 32 consecutive samples then their plus
 // sides, so every warp traces one side along one edge (same behaviour per lane).
@@ -1063,7 +1067,11 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
                      !(s->lbin_total_host && *s->lbin_total_host > s->lbin_cap);
     if (!p.lbins_reused) s->lbins_valid = false;
   }
-  p.hz = p.total >= (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN) && p.total >= (long long)HZ_JOBS_PER_FACE * s->nf;
+  {
+    const bool unlisted = s->env.w > 0 || p.max_vl > 0 || (s->nl > 0 && !p.lbins);
+    const double rays = (p.B - 1) + (unlisted ? p.B : 0.25);   // per path
+    p.hz = p.total >= (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN) && rays * (double)p.total >= (double)HZ_GAIN * s->nf;
+  }
   p.hz_reused = p.hz && s->hz_valid && s->hz_geom == s->geom_version;
   if (p.hz && !p.hz_reused) s->hz_valid = false;
   if (p.kind == 0 && p.pixels > s->acc_cap) {
