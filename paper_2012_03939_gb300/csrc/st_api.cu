@@ -1328,14 +1328,15 @@ st_status st_scene_create(const st_scene_desc* d, void* stream, st_scene** out) 
   chk(dalloc(&s->keys, (size_t)n)); chk(dalloc(&s->keys2, (size_t)n)); chk(dalloc(&s->ids, (size_t)n));
   chk(dalloc(&s->ids2, (size_t)n)); chk(dalloc(&s->hist, 256 * (size_t)s->sort_blocks)); chk(dalloc(&s->bounds, 6));
   chk(dalloc(&s->nodes4, 7 * (size_t)std::max(n - 1, 1))); chk(dalloc(&s->src4, 4 * (size_t)std::max(n - 1, 1)));
-  chk(dalloc(&s->q4, 4 * (size_t)n)); chk(dalloc(&s->c4, 2));
+  chk(dalloc(&s->q4, 4 * (size_t)n)); chk(dalloc(&s->c4, 3));
   chk(dalloc(&s->lights, 2 * (size_t)std::max(s->nl, 1))); chk(dalloc(&s->edge_v, ev.size()));
   chk(dalloc(&s->edge_f, ef.size())); chk(dalloc(&s->d_args, 1)); chk(dalloc(&s->d_err, 1));
   chk(dalloc(&s->mstat, 1));
   {
     const size_t m4 = (size_t)std::max(n - 1, 1);
     chk(dalloc(&s->parent4, m4)); chk(dalloc(&s->leaf_node4, (size_t)n));
-    chk(dalloc(&s->hz, (size_t)n)); chk(dalloc(&s->hz_nodes, 3 * m4)); chk(dalloc(&s->hz_done, m4));
+    // one record more than there are nodes: the hierarchy's build takes hz and hz_nodes as scratch
+    chk(dalloc(&s->hz, (size_t)n)); chk(dalloc(&s->hz_nodes, 3 * m4 + 1)); chk(dalloc(&s->hz_done, m4));
   }
   {
     // edge hierarchy: at most 2^14 leaf blocks of at least 4 edges

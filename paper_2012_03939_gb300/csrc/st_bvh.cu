@@ -387,6 +387,59 @@ __global__ void __launch_bounds__(SCAN2_BLOCK) k_ploc_merge(const int* nn, int c
   }
 }
 
+// The last rounds, from at most SCAN2_BLOCK clusters down to the root, in one block that holds them in shared memory
+// (the same neighbours, flags and positions as the kernels above). A round there costs four launches and a read of its
+// counts by the host, some 35 us whatever its size, and about half of a build's rounds have fewer clusters than one
+// block has threads; here it is bounded by the block's own barriers and shared-memory reads, a few us.
+// status = (1 when the root is reached, clusters left).
+// With the collapse's small levels in one block (k_collapse_few) and no allocation per call, a rebuild of the 50k-face
+// torus knot and a trace of 65536 rays went from 2049 to 1160 us on one GB300.
+__global__ void __launch_bounds__(SCAN2_BLOCK) k_ploc_tail(const int* cid, const float4* lo, const float4* hi, int c,
+                                                          int next, int n, float4* nodes, int* parent, int2* status) {
+  __shared__ float4 slo[SCAN2_BLOCK], shi[SCAN2_BLOCK];
+  __shared__ int sid[SCAN2_BLOCK], nn[SCAN2_BLOCK];
+  __shared__ int2 sh[32];
+  const int i = threadIdx.x;
+  if (i < c) { slo[i] = lo[i]; shi[i] = hi[i]; sid[i] = cid[i]; }
+  __syncthreads();
+  while (c > 1) {   // a round without a merge ends the loop, so it runs fewer than SCAN2_BLOCK times
+    float4 al = make_float4(0, 0, 0, 0), ah = al;
+    if (i < c) {
+      al = slo[i]; ah = shi[i];
+      float best = __int_as_float(0x7f800000);
+      int bj = -1;
+      for (int j = max(i - PLOC_R, 0); j <= min(i + PLOC_R, c - 1); ++j) {
+        if (j == i) continue;
+        float a = merged_area(al, ah, slo[j], shi[j]);
+        if (a < best) { best = a; bj = j; }
+      }
+      nn[i] = bj;
+    }
+    __syncthreads();
+    const int2 f = i < c ? ploc_flags(nn, i) : make_int2(0, 0);
+    int2 tot;
+    const int2 pos = block_scan2(f, sh, tot);
+    if (tot.x <= 0 || tot.y != c - tot.x) break;   // uniform: non-finite boxes
+    int id = i < c ? sid[i] : 0;
+    if (f.x) {
+      const int j = nn[i], k = next - 1 - pos.x, b = sid[j];
+      const float4 bl = slo[j], bh = shi[j];
+      nodes[4 * k + 3] = make_float4(__int_as_float(id), __int_as_float(b), 0.0f, 0.0f);
+      if (id >= 0) parent[id] = k; else parent[(n - 1) + ~id] = k;
+      if (b >= 0) parent[b] = k; else parent[(n - 1) + ~b] = k;
+      id = k;
+      al = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.0f);
+      ah = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), 0.0f);
+    }
+    __syncthreads();
+    if (f.y) { sid[pos.y] = id; slo[pos.y] = al; shi[pos.y] = ah; }
+    next -= tot.x;
+    c = tot.y;
+    __syncthreads();
+  }
+  if (i == 0) *status = make_int2(c == 1 && next == 0 ? 1 : 0, c);
+}
+
 namespace {
 cudaError_t morton_order(st_scene* s, cudaStream_t stream) {
   int n = s->nf;
@@ -423,23 +476,21 @@ cudaError_t bvh_build_ploc(st_scene* s, cudaStream_t stream) {
   int n = s->nf;
   cudaError_t e = morton_order(s, stream);
   if (e != cudaSuccess || n < 2) return e != cudaSuccess ? e : boxes(s, stream);
-  // scratch for the rounds: two cluster arrays (box, id), scans, neighbours
-  int nb = (n + SCAN2_BLOCK - 1) / SCAN2_BLOCK;
-  size_t bytes = 4 * (size_t)n * sizeof(float4) + (size_t)n * sizeof(int2) + (size_t)(nb + 1) * sizeof(int2) +
-                 3 * (size_t)n * sizeof(int);
-  char* buf = nullptr;
-  e = cudaMalloc((void**)&buf, bytes);
-  if (e != cudaSuccess) return e;
-  float4* lo[2] = {(float4*)buf, (float4*)buf + n};
-  float4* hi[2] = {(float4*)buf + 2 * (size_t)n, (float4*)buf + 3 * (size_t)n};
-  int2* scan = (int2*)((float4*)buf + 4 * (size_t)n);
-  int2* part = scan + n;
-  int* cid[2] = {(int*)(part + nb + 1), (int*)(part + nb + 1) + n};
-  int* nn = cid[1] + n;
+  // Scratch for the rounds: two cluster arrays (box, id), scans, neighbours. All of it is the scene's own memory whose
+  // content the build makes stale or has used already: the free directions (4 n - 2 float4), the collapse's queues (4 n
+  // ints) and the sort's keys and second buffers (n ints each). Allocated per call it cost an allocation, a
+  // synchronisation and a release.
+  float4* hzn = s->hz_nodes;
+  float4* lo[2] = {reinterpret_cast<float4*>(s->hz), hzn + n};   // n, n - 1
+  float4* hi[2] = {hzn, hzn + 2 * (size_t)n - 1};                // n, n - 1
+  int2* scan = reinterpret_cast<int2*>(s->q4);
+  int2* part = scan + n;   // of n / SCAN2_BLOCK blocks and the total: at most n
+  int* cid[2] = {reinterpret_cast<int*>(s->keys2), s->ids2};
+  int* nn = reinterpret_cast<int*>(s->keys);
   k_ploc_init<<<(n + 255) / 256, 256, 0, stream>>>(s->verts, s->faces, s->ids, n, cid[0], lo[0], hi[0]);
   int c = n, next = n - 1, cur = 0;
   int2 tot = make_int2(0, 0);
-  for (int round = 0; c > 1 && e == cudaSuccess; ++round) {
+  for (int round = 0; c > SCAN2_BLOCK && e == cudaSuccess; ++round) {
     if (round > 4 * n) { e = cudaErrorIllegalState; break; }
     int g = (c + PLOC_BLOCK - 1) / PLOC_BLOCK, gs = (c + SCAN2_BLOCK - 1) / SCAN2_BLOCK;
     k_ploc_nn<<<g, PLOC_BLOCK, 0, stream>>>(lo[cur], hi[cur], c, nn);
@@ -457,12 +508,14 @@ cudaError_t bvh_build_ploc(st_scene* s, cudaStream_t stream) {
     c = tot.y;
     cur ^= 1;
   }
-  if (e == cudaSuccess && next != 0) e = cudaErrorIllegalState;
+  if (e != cudaSuccess) return e;
+  k_ploc_tail<<<1, SCAN2_BLOCK, 0, stream>>>(cid[cur], lo[cur], hi[cur], c, next, n, s->nodes, s->parent, part);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&tot, part, sizeof(int2), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->parent, 0xff, sizeof(int), stream);   // the root has no parent
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  cudaFree(buf);
-  if (e != cudaSuccess) return e;
-  return boxes(s, stream);
+  if (e == cudaSuccess && tot.x != 1) e = cudaErrorIllegalState;
+  return e != cudaSuccess ? e : boxes(s, stream);
 }
 
 // ---- 4-wide collapse: each 4-wide node takes a binary node's children and
@@ -479,10 +532,9 @@ __device__ __forceinline__ float binary_area(const float4* nodes, int c) {
 
 constexpr int EMPTY4 = (int)0x80000000;
 
-__global__ void k_collapse(const float4* nodes, const int* qin, int nin, int* qout, int* counters, int* src4,
-                           float4* nodes4, int* parent4, int* leaf_node4) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nin) return;
+// entry k of the queue: its node, and its internal children into the next queue (counters: nodes so far, entries there)
+__device__ __forceinline__ void collapse_entry(const float4* nodes, const int* qin, int k, int* qout, int* counters,
+                                               int* src4, float4* nodes4, int* parent4, int* leaf_node4) {
   int b = qin[2 * k], id = qin[2 * k + 1];
   float4 n3 = nodes[4 * b + 3];
   int slot[4] = {__float_as_int(n3.x), __float_as_int(n3.y), EMPTY4, EMPTY4};
@@ -518,6 +570,38 @@ __global__ void k_collapse(const float4* nodes, const int* qin, int nin, int* qo
   }
   nodes4[7 * id + 6] = make_float4(__int_as_float(child[0]), __int_as_float(child[1]), __int_as_float(child[2]),
                                    __int_as_float(child[3]));
+}
+
+__global__ void k_collapse(const float4* nodes, const int* qin, int nin, int* qout, int* counters, int* src4,
+                           float4* nodes4, int* parent4, int* leaf_node4) {
+  int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < nin) collapse_entry(nodes, qin, k, qout, counters, src4, nodes4, parent4, leaf_node4);
+}
+
+// Levels of at most COLLAPSE_FEW entries, one after the other in one block: the first five or six, and the last ones of
+// a tree whose depth is uneven. A level of its own costs a launch and a read of its count by the host, about 25 us.
+// counters = (nodes so far, entries of the queue it stopped at, levels done).
+constexpr int COLLAPSE_FEW = 1024, COLLAPSE_LEVELS = 64;
+__global__ void __launch_bounds__(COLLAPSE_FEW) k_collapse_few(const float4* nodes, int* qa, int* qb, int nin, int first,
+                                                              int levels, int* counters, int* src4, float4* nodes4, int* parent4,
+                                                              int* leaf_node4) {
+  __shared__ int cnt[2];
+  const int t = threadIdx.x;
+  if (t == 0) {
+    cnt[0] = first ? 1 : counters[0];
+    if (first) { qa[0] = 0; qa[1] = 0; parent4[0] = -1; }   // binary root -> 4-wide node 0
+  }
+  int level = 0;
+  for (; nin > 0 && nin <= COLLAPSE_FEW && level < levels; ++level) {
+    if (t == 0) cnt[1] = 0;
+    __syncthreads();
+    if (t < nin) collapse_entry(nodes, qa, t, qb, cnt, src4, nodes4, parent4, leaf_node4);
+    __syncthreads();
+    nin = cnt[1];
+    int* q = qa; qa = qb; qb = q;
+    __syncthreads();
+  }
+  if (t == 0) { counters[0] = cnt[0]; counters[1] = nin; counters[2] = level; }
 }
 
 // child boxes of every 4-wide node from the binary boxes / leaf triangles
@@ -564,25 +648,31 @@ cudaError_t bvh_collapse(st_scene* s, cudaStream_t stream) {
   int n = s->nf;
   s->n4 = 0;
   if (n < 2) return cudaSuccess;
-  int init[2] = {0, 0};   // binary root -> 4-wide node 0
-  int cnt[2] = {1, 0};
+  int cnt[3] = {1, 0, 1};
   int* qa = s->q4;
   int* qb = s->q4 + 2 * (size_t)n;
-  cudaError_t e = cudaMemcpyAsync(qa, init, sizeof(init), cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s->c4, cnt, sizeof(cnt), cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->parent4, 0xff, sizeof(int), stream);   // the root has no parent
+  cudaError_t e = cudaSuccess;
   int nin = 1;
-  for (int level = 0; nin > 0 && e == cudaSuccess; ++level) {
-    if (level > 64) return cudaErrorIllegalState;  // deeper than any tree built here: malformed
-    e = cudaMemsetAsync(s->c4 + 1, 0, sizeof(int), stream);
-    if (e != cudaSuccess) break;
-    k_collapse<<<(nin + 127) / 128, 128, 0, stream>>>(s->nodes, qa, nin, qb, s->c4, s->src4, s->nodes4,
-                                                    s->parent4, s->leaf_node4);
+  for (int level = 0; nin > 0 && e == cudaSuccess;) {
+    if (level > COLLAPSE_LEVELS) return cudaErrorIllegalState;  // deeper than any tree built here: malformed
+    const bool few = nin <= COLLAPSE_FEW;
+    if (few) {
+      k_collapse_few<<<1, COLLAPSE_FEW, 0, stream>>>(s->nodes, qa, qb, nin, level == 0 ? 1 : 0,
+                                                     COLLAPSE_LEVELS + 1 - level, s->c4, s->src4, s->nodes4, s->parent4,
+                                                     s->leaf_node4);
+    } else {
+      e = cudaMemsetAsync(s->c4 + 1, 0, sizeof(int), stream);
+      if (e != cudaSuccess) break;
+      k_collapse<<<(nin + 127) / 128, 128, 0, stream>>>(s->nodes, qa, nin, qb, s->c4, s->src4, s->nodes4, s->parent4,
+                                                        s->leaf_node4);
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, s->c4, sizeof(cnt), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     nin = cnt[1];
-    std::swap(qa, qb);
+    const int done = few ? cnt[2] : 1;
+    level += done;
+    if (done & 1) std::swap(qa, qb);
   }
   if (e != cudaSuccess) return e;
   s->n4 = cnt[0];

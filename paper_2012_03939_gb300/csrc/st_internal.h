@@ -131,7 +131,7 @@ struct st_scene {
   float4* nodes4 = nullptr;      // [n4*7]: lo.x[4], hi.x[4], lo.y[4], hi.y[4], lo.z[4], hi.z[4], children[4]
   int* src4 = nullptr;           // [n4*4]: binary node (>= 0) or ~leaf (< 0) behind each child slot
   int* q4 = nullptr;             // [4*F] collapse work queues
-  int* c4 = nullptr;             // [2] collapse counters
+  int* c4 = nullptr;             // [3] collapse counters
   int n4 = 0;
   // lights
   float4* lights = nullptr;      // [nl*2]: (pos, 0), (intensity, 0)
