@@ -76,6 +76,15 @@ constexpr double BIN_FACES_PER_CELL = 0.5;
 // below HZ_MIN_JOBS_OPEN.
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
 constexpr int HZ_GAIN = 200;
+// A forward call that no adjoint follows has to win the build back by itself. On gentle surfaces it does from HZ_GAIN on
+// (two-view preview of 200k faces, 250 rays a face: 5.5 -> 4.9 ms); on rough or concave ones a build costs twice as much
+// and spares half: renders alone, with and without the build, of 1M rough faces (300 rays a face) 39.2 and 27.2 ms, of
+// 249k (315) 12.2 and 11.0, of a 50k-face torus knot (1170) 4.60 and 4.39; of one of 36k faces (4200) 7.65 with, 8.75
+// before there were any. So HZ_GAIN_ROUGH is asked of these. The surface is gentle while the sines by which neighbours
+// rise above a face average below HZ_GENTLE (displaced spheres 0 to 2e-5, torus knot 0.0097, rough 0.022), as the scene
+// was created; an adjoint follows if one did on these vertices or the last.
+constexpr int HZ_GAIN_ROUGH = 1600;
+constexpr double HZ_GENTLE = 0.002;
 // Segment bases and chunk sizes are multiples of 64: an edge segment is laid out
 // in blocks of 64 jobs, the minus sides of 32 consecutive samples then their plus
 // sides, so every warp traces one side along one edge (same behaviour per lane).
@@ -199,6 +208,40 @@ void build_edges(const std::vector<int>& F, int nf, std::vector<int2>& ev, std::
     ef.push_back(make_int2(e[i].second, second));
     i = j;
   }
+}
+
+// Mean over the edges of two faces of the sine by which the second face rises above the plane of the first, on the
+// outer side of a closed mesh (0 where it falls away).
+double mean_rise(const std::vector<float>& V, const std::vector<int>& F, int nf, const std::vector<int2>& ev,
+                 const std::vector<int2>& ef) {
+  auto at = [&](int v, double (&x)[3]) { for (int k = 0; k < 3; ++k) x[k] = V[3 * (size_t)v + k]; };
+  auto normal = [&](int f, double (&n)[3], double (&a)[3]) {
+    double b[3], c[3];
+    at(F[3 * f], a); at(F[3 * f + 1], b); at(F[3 * f + 2], c);
+    for (int k = 0; k < 3; ++k) { b[k] -= a[k]; c[k] -= a[k]; }
+    for (int k = 0; k < 3; ++k) n[k] = b[(k + 1) % 3] * c[(k + 2) % 3] - b[(k + 2) % 3] * c[(k + 1) % 3];
+  };
+  auto len = [](const double (&x)[3]) { return std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]); };
+  double vol = 0.0, n[3], a[3];
+  for (int f = 0; f < nf; ++f) {
+    normal(f, n, a);
+    vol += n[0] * a[0] + n[1] * a[1] + n[2] * a[2];
+  }
+  double sum = 0.0;
+  size_t cnt = 0;
+  for (size_t i = 0; i < ef.size(); ++i) {
+    if (ef[i].y < 0) continue;
+    const int* g = &F[3 * (size_t)ef[i].y];
+    const int apex = g[0] != ev[i].x && g[0] != ev[i].y ? g[0] : g[1] != ev[i].x && g[1] != ev[i].y ? g[1] : g[2];
+    double x[3], b[3];
+    normal(ef[i].x, n, a);
+    at(apex, x); at(ev[i].x, b);
+    for (int k = 0; k < 3; ++k) x[k] -= b[k];
+    const double h = (vol < 0.0 ? -1.0 : 1.0) * (n[0] * x[0] + n[1] * x[1] + n[2] * x[2]), l = len(n) * len(x);
+    if (h > 0.0 && l > 0.0) sum += h / l;
+    ++cnt;
+  }
+  return cnt ? sum / (double)cnt : 0.0;
 }
 
 // True when the faces form one connected surface (across shared edges) in
@@ -1070,7 +1113,14 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
   {
     const bool unlisted = s->env.w > 0 || p.max_vl > 0 || (s->nl > 0 && !p.lbins);
     const double rays = (p.B - 1) + (unlisted ? p.B : 0.25);   // per path
-    p.hz = p.total >= (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN) && rays * (double)p.total >= (double)HZ_GAIN * s->nf;
+    const bool built = s->hz_valid && s->hz_geom == s->geom_version;
+    const bool alone = p.kind == 0 && !built && !s->gentle && !(s->adj_seen && s->geom_version - s->adj_geom <= 1);
+    p.hz = p.total >= (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN) &&
+           rays * (double)p.total >= (double)(alone ? HZ_GAIN_ROUGH : HZ_GAIN) * s->nf;
+    if (p.kind == 1) {
+      s->adj_seen = true;
+      s->adj_geom = s->geom_version;
+    }
   }
   p.hz_reused = p.hz && s->hz_valid && s->hz_geom == s->geom_version;
   if (p.hz && !p.hz_reused) s->hz_valid = false;
@@ -1295,6 +1345,7 @@ st_status st_scene_create(const st_scene_desc* d, void* stream, st_scene** out) 
   std::vector<int2> ev, ef;
   build_edges(hf, s->nf, ev, ef);
   s->closed = closed_single_surface(hf, s->nf, ef);
+  s->gentle = mean_rise(hv, hf, s->nf, ev, ef) < HZ_GENTLE;
   s->n_edges = (int)ev.size();
   std::vector<float4> etex;
   std::vector<float2> etab;

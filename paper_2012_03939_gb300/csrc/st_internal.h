@@ -194,6 +194,9 @@ struct st_scene {
   cudaEvent_t hz_ev[2] = {};               // its fork and join
   bool hz_valid = false;
   unsigned long long hz_geom = 0;
+  bool gentle = false;           // neighbouring faces hardly rise above one another (mean_rise)
+  bool adj_seen = false;         // geom_version of the last adjoint call
+  unsigned long long adj_geom = 0;
   float* acc = nullptr;          // [6 * pixels] forward accumulation, compensated FP32 (sum, error) per channel
   unsigned long long* sacc = nullptr;  // [pixels] path-signature sums (bin-space pixel index)
   long long acc_cap = 0;

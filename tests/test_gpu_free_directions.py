@@ -76,6 +76,8 @@ def test_free_directions_change_nothing(st, mesh, light, smooth):
                  views=views, max_bounces=4, smooth_normals=smooth)
     scene = st.Scene.from_scene(sc)
     sig = torch.zeros(sc.n_pixels, dtype=torch.int64, device="cuda")
+    # an adjoint builds them on rough and concave meshes too, where a forward call alone would not
+    scene.backward(sc.views, 4, 5, torch.zeros((sc.n_pixels, 3), device="cuda"))
     img = scene.render(sc.views, 4, 5, signatures=sig).cpu().numpy()
     stats = scene.stats()
     paths = sum(v.width * v.height * v.spp for v in views)
