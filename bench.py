@@ -626,7 +626,7 @@ def run_ours(args):
                      "shadow_ms": round(a["shadow_ms"] + b["shadow_ms"], 3), "graph": False,
                      "chunks_overlapped": False,
                      "note": "kernels timed one by one on one stream; the timed step overlaps consecutive chunks on "
-                             "two engines and streams (ms_per_step)"}
+                             "up to four engines and streams (ms_per_step)"}
 
     # end to end through the C ABI with host buffers: H2D of the mesh state and
     # D2H of the image and both gradients every step
