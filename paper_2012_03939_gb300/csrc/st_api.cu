@@ -961,8 +961,11 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
   return ST_OK;
 }
 
+// What a captured call depends on besides the tables it reads from device memory: a replay takes every launch size and
+// scalar argument as captured. n4 is one of them (traversal's bounds, the free directions' build), and a rebuild of the
+// hierarchy changes it.
 std::vector<long long> graph_key(const Plan& p, int Q, const st_scene* s) {
-  std::vector<long long> k = {p.kind, p.B, (long long)p.views.size(), Q, p.o.edge_term, p.o.edge_mode, p.o.edge_spp,
+  std::vector<long long> k = {s->n4, p.kind, p.B, (long long)p.views.size(), Q, p.o.edge_term, p.o.edge_mode, p.o.edge_spp,
                               p.interior, p.edges, p.o.count_visits, p.bins, p.cull, p.bins_reused, p.lbins,
                               p.lbins_reused, s->lbin_cap,
                               p.o.persist_blocks, s->bin_cap, p.max_vl, p.sig, p.sec_tree, p.hz, p.hz_reused,
