@@ -35,10 +35,10 @@ __host__ __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x 
 __host__ __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
   return mk3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
-__device__ __forceinline__ float len3(float3 a) { return sqrtf(dot3(a, a)); }
-__device__ __forceinline__ float3 norm3(float3 a) { float l = len3(a); return mk3(a.x / l, a.y / l, a.z / l); }
-__device__ __forceinline__ float3 xyz(float4 a) { return mk3(a.x, a.y, a.z); }
-__device__ __forceinline__ float comp3(float3 a, int k) { return k == 0 ? a.x : (k == 1 ? a.y : a.z); }
+__host__ __device__ __forceinline__ float len3(float3 a) { return sqrtf(dot3(a, a)); }
+__host__ __device__ __forceinline__ float3 norm3(float3 a) { float l = len3(a); return mk3(a.x / l, a.y / l, a.z / l); }
+__host__ __device__ __forceinline__ float3 xyz(float4 a) { return mk3(a.x, a.y, a.z); }
+__host__ __device__ __forceinline__ float comp3(float3 a, int k) { return k == 0 ? a.x : (k == 1 ? a.y : a.z); }
 
 // ------------------------------------------------------------------ Philox4x32-10
 // Counter-based generator of Salmon et al. (SC'11): ten rounds of two 32x32
@@ -132,7 +132,7 @@ struct RayPre {
   float sx, sy, sz;
 };
 
-__device__ __forceinline__ RayPre ray_pre(float3 o, float3 d) {
+__host__ __device__ __forceinline__ RayPre ray_pre(float3 o, float3 d) {
   RayPre r;
   r.o = o;
   float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
@@ -149,7 +149,7 @@ __device__ __forceinline__ RayPre ray_pre(float3 o, float3 d) {
 }
 
 // returns t (> T_EPS and < tmax) or a negative value on a miss
-__device__ __forceinline__ float tri_test(const RayPre& r, float3 p0, float3 p1, float3 p2, float tmax) {
+__host__ __device__ __forceinline__ float tri_test(const RayPre& r, float3 p0, float3 p1, float3 p2, float tmax) {
   float3 A = p0 - r.o, B = p1 - r.o, C = p2 - r.o;
   float Akz = comp3(A, r.kz), Bkz = comp3(B, r.kz), Ckz = comp3(C, r.kz);
   float Ax = comp3(A, r.kx) - r.sx * Akz, Ay = comp3(A, r.ky) - r.sy * Akz;

@@ -34,14 +34,16 @@
 // then seen from f along t d + e + eta: with rho = (|e| + eta) / T_EPS and e_n the
 // part of e along n, its sine of elevation is at least (d_n - (eta - e_n) / T_EPS)
 // / (1 + rho) (e_n < 0) and at most (d_n + (eta + e_n) / T_EPS) / (1 - rho) (e_n >
-// 0), its azimuth off by about rho / |d_h|, which the widened sectors cover up to
-// HZ_WIDEN; past that every sector counts. A ray in the plane of a neighbour that
+// 0), its azimuth off by up to asin((rho + HZ_TILT) / |d_h|), which the widened
+// sectors cover up to HZ_WIDEN; past that every sector counts. A ray in the plane of a neighbour that
 // runs off its far side can still be given a false hit (the neighbour's projection
 // is a line through the origin, its weights are rounding, and t any depth of its
-// vertices): p is then within eta / d_n of the shared edge, so a direction must
-// also be steeper than eta / w, w the distance of p to f's nearest edge. (Of 6 10^8
-// sampled free rays, half from within 10^-5 of an edge's length of it, one had such a
-// hit without this; of 3.4 10^9 none has with it, over twelve meshes.)
+// vertices): p is then within (|e| + eta) / d_n of the shared edge, so a direction
+// must also be steeper than (|e| + eta) / w, w the distance of p to f's nearest edge.
+// (Of 6 10^8 sampled free rays, half from within 10^-5 of an edge's length of it, one
+// had such a hit without this. With it: none of 3.4 10^9 over twelve meshes about the
+// origin, and of 7.7 10^9 rays from a face to one neighbour, coordinates up to 10^4 and
+// faces from 10^-3 to 5, no free one hit; with eta / w alone one did, at 10^3.)
 //
 // Measured on one GB300. k_horizon is bounded by instruction issue (55 % active, 16 to
 // 24 warps per SM, 15 of 32 lanes: nodes and triangles of a round take different
@@ -55,12 +57,16 @@
 // 200k-face iteration went from 31.4 to 30.0, one of 32 captures lit from the camera
 // from 5.76 to 5.29, both on the later kernels.)
 #pragma once
+#include <cmath>
+
 #include "st_internal.h"
 #include "st_trace.cuh"
 
 namespace st {
 
 constexpr float HZ_WIDEN = 0.1f;      // radians added to each side of a sector
+constexpr float HZ_SIN = 0.0998f;     // its sine, rounded down: what an uncertain azimuth may be off by
+constexpr float HZ_TILT = 4e-4f;      // a direction's offset from the rounding of a face's normal (slivers up to hz_face's limit)
 constexpr float HZ_RHO = 4.0f;        // largest rho for which the directions are used
 constexpr float HZ_MARGIN = 0.003f;   // constant part of the elevation margin (rounding of the frames)
 constexpr float HZ_FLOOR = 0.003f;    // sine of elevation below which nothing is free
@@ -72,7 +78,7 @@ constexpr int HZ_STACK = 96;          // nodes waiting to be opened; one past th
 constexpr int HZ_OPEN = 512;          // nodes opened per face, likewise
 
 // position of a sine of elevation among the 16 bands: [HZ_FLOOR, HZ_LOW), then 15 of equal width up to 1
-__device__ __forceinline__ float hz_band(float s) {
+__host__ __device__ __forceinline__ float hz_band(float s) {
   return s < HZ_LOW ? (s - HZ_FLOOR) * (1.0f / (HZ_LOW - HZ_FLOOR)) : 1.0f + (s - HZ_LOW) * (15.0f / (1.0f - HZ_LOW));
 }
 
@@ -97,7 +103,7 @@ __host__ __device__ constexpr HzLines hz_lines() {
 }
 
 // Sectors that hold some w whose products with the border normals and axes lie in [lo, hi].
-__device__ __forceinline__ unsigned hz_sectors(const float (&blo)[8], const float (&bhi)[8], const float (&clo)[4],
+__host__ __device__ __forceinline__ unsigned hz_sectors(const float (&blo)[8], const float (&bhi)[8], const float (&clo)[4],
                                                const float (&chi)[4], float tiny) {
   unsigned m = 0;
 #pragma unroll
@@ -114,15 +120,24 @@ __device__ __forceinline__ unsigned hz_sectors(const float (&blo)[8], const floa
 
 // Square root to a few units in the last place (0 for what rounding left below it): the bounds built from it carry
 // wider margins (1e-5 relative).
-__device__ __forceinline__ float hz_sqrt(float x) {
+__host__ __device__ __forceinline__ float hz_sqrt(float x) {
   x = fmaxf(x, 1e-30f);
   return x * rsqrtf(x);
 }
 
+// a / b to a few units in the last place
+__host__ __device__ __forceinline__ float hz_div(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(a, b);
+#else
+  return a / b;
+#endif
+}
+
 // arctangent of y / x over the full circle within 4e-3 rad (Rajan et al., "Efficient approximations for the
 // arctangent function", IEEE Signal Processing Magazine 2006, eq. 5: pi/4 t + 0.273 t (1 - t) on [0, 1])
-__device__ __forceinline__ float hz_atan2(float y, float x) {
-  const float ax = fabsf(x), ay = fabsf(y), t = __fdividef(fminf(ax, ay), fmaxf(fmaxf(ax, ay), 1e-30f));
+__host__ __device__ __forceinline__ float hz_atan2(float y, float x) {
+  const float ax = fabsf(x), ay = fabsf(y), t = hz_div(fminf(ax, ay), fmaxf(fmaxf(ax, ay), 1e-30f));
   float a = t * (1.05839816f - 0.273f * t);   // pi / 4 + 0.273
   if (ay > ax) a = 1.57079633f - a;
   if (x < 0.0f) a = PI_F - a;
@@ -206,7 +221,8 @@ __global__ void k_hz_nodes(const float4* __restrict__ nodes, const float4* __res
         }
       }
     }
-    q.R = fminf(r, 0.5f * len3(hi - lo)) * 1.00001f;
+    const float3 up = hi - q.c, dn = q.c - lo;   // the centre is rounded: the box's corners are as far as this from it
+    q.R = fminf(r, len3(mk3(fmaxf(up.x, dn.x), fmaxf(up.y, dn.y), fmaxf(up.z, dn.z)))) * 1.00001f;
     q.smax = fminf(smax, q.R);
     q.smin = fmaxf(smin, -q.R);
     __stcg(&N[3 * k], make_float4(q.c.x, q.c.y, q.c.z, q.R));
@@ -224,6 +240,162 @@ __global__ void k_hz_nodes(const float4* __restrict__ nodes, const float4* __res
   atomicOr(err, ERR_LOOP);
 }
 
+// A face as its directions are seen from: frame, centre and radius. Positions are taken from the vertex v0 (c too): near
+// the face such differences of floats are exact or nearly so, wherever it lies, while a centroid of absolute coordinates
+// is off by an ulp of these, which on a small face far from the origin is more than what its neighbours rise by.
+struct HzFace {
+  float3 v0, v1, v2, n, T, B, c;
+  float r, tiny;
+};
+// False on a sliver, whose normal and borders are not known well enough: nothing is free on it.
+__host__ __device__ __forceinline__ bool hz_face(float3 v0, float3 v1, float3 v2, float side, HzFace& f) {
+  const float3 e1 = v1 - v0, e2 = v2 - v0;
+  const float3 m = cross3(e1, e2);
+  const float l1 = len3(e1), l2 = len3(e2), l3 = len3(v2 - v1), ml = len3(m);
+  const float lmax = fmaxf(l1, fmaxf(l2, l3));
+  if (!(ml > 1e-3f * lmax * lmax) || !(l1 > 1e-3f * lmax)) return false;
+  f.v0 = v0; f.v1 = v1; f.v2 = v2;
+  f.n = m * (side / ml);
+  f.T = e1 * (1.0f / l1);
+  f.B = cross3(f.n, f.T);
+  f.c = (e1 + e2) * (1.0f / 3.0f);
+  f.r = fmaxf(len3(f.c), fmaxf(len3(e1 - f.c), len3(e2 - f.c)));
+  f.tiny = 1e-6f * fminf(lmax, 1.0f);
+  return true;
+}
+// f in its plane: the border lines (mx, my, mo) of vertex k (0 .. 2), m the outward normal (f runs clockwise about n
+// when side < 0) of the edge that starts there (line k) and its bisector with the edge that ends there (line 3 + k).
+__host__ __device__ __forceinline__ void hz_border(const HzFace& f, float side, int k, float* ln) {
+  auto in2 = [&](int i) { float3 d = (i == 0 ? f.v0 : i == 1 ? f.v1 : f.v2) - f.v0; return make_float2(dot3(d, f.T), dot3(d, f.B)); };
+  const float2 p0 = in2(k), p1 = in2(k == 2 ? 0 : k + 1), p2 = in2(k == 0 ? 2 : k - 1);
+  auto normal = [&](float2 a, float2 b) {
+    float dx = b.x - a.x, dy = b.y - a.y, il = side / sqrtf(dx * dx + dy * dy);
+    return make_float2(dy * il, -dx * il);
+  };
+  const float2 m0 = normal(p0, p1), m1 = normal(p2, p0);   // of the edges that start and end at vertex k
+  ln[k] = m0.x; ln[6 + k] = m0.y;
+  const auto out = [&](float mx, float my) {   // the least mo with m.y <= mo on all of f
+    return fmaxf(mx * p0.x + my * p0.y, fmaxf(mx * p1.x + my * p1.y, mx * p2.x + my * p2.y));
+  };
+  ln[12 + k] = out(m0.x, m0.y);
+  const float sx = m0.x + m1.x, sy = m0.y + m1.y, il = rsqrtf(fmaxf(sx * sx + sy * sy, 1e-12f));
+  ln[3 + k] = sx * il; ln[9 + k] = sy * il;
+  ln[15 + k] = out(sx * il, sy * il);
+}
+
+// Marked cells: sector 2 w in the low half of word w, 2 w + 1 in the high.
+struct HzCells { unsigned w[4]; };
+// the cells of elevations lo .. hi in the sectors sec
+__host__ __device__ __forceinline__ HzCells hz_cells(unsigned sec, float lo, float hi) {
+  HzCells c;
+  int b0 = (int)floorf(hz_band(lo) - 1e-3f), b1 = (int)floorf(hz_band(hi) + 1e-3f);
+  b0 = b0 > 0 ? b0 : 0;
+  b1 = b1 < 15 ? b1 : 15;
+  unsigned m = b1 >= b0 ? (2u << b1) - (1u << b0) : 0u;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) c.w[w] = (sec >> (2 * w) & 1u ? m : 0u) | (sec >> (2 * w + 1) & 1u ? m << 16 : 0u);
+  return c;
+}
+// cells of points within r of f's centre + v, at most hb high; far: small enough to be taken so
+__host__ __device__ __forceinline__ HzCells hz_sphere(const HzFace& f, float3 v, float r, float hb, bool& far) {
+  const float d2 = dot3(v, v), vn = dot3(v, f.n), vx = dot3(v, f.T), vy = dot3(v, f.B);
+  unsigned sec = 0xffu;
+  float lo = -1.0f, hi = 1.0f;
+  far = false;
+  if (r * r < d2) {
+    const float iv = rsqrtf(d2), sv = vn * iv, sr = r * iv, cv = hz_sqrt(1.0f - sv * sv),
+                cr = hz_sqrt(1.0f - sr * sr);
+    if (cv >= sr || sv < 0.0f) hi = sv * cr + cv * sr + 1e-4f;
+    if (cv >= sr || sv > 0.0f) lo = sv * cr - cv * sr - 1e-4f;
+    const float D = hz_sqrt(vx * vx + vy * vy) * 0.99999f - r;
+    if (D > 0.0f) {
+      hi = fminf(hi, hb * rsqrtf(D * D + hb * hb) * 1.00001f);
+      // azimuth of the centre and of its disk, in sectors: asin x <= x + (pi / 2 - 1) x^3 on [0, 1]
+      const float x = hz_div(r, D + r), a = hz_atan2(vy, vx) * (4.0f / PI_F),
+                  w = (x + 0.5708f * x * x * x + HZ_WIDEN + 5e-3f) * (4.0f / PI_F);
+      const int s0 = (int)floorf(a - w), n = (int)floorf(a + w) - s0 + 1;
+      if (n < 8) {
+        const unsigned m = (1u << n) - 1u, t = (unsigned)s0 & 7u;
+        sec = (m << t | m >> (8u - t)) & 0xffu;
+      }
+    }
+    far = sr < HZ_FAR;
+  }
+  return hz_cells(sec, lo, hi);
+}
+// a triangle's sphere about its own centre (v from f's) and how high it reaches over f's plane
+__host__ __device__ __forceinline__ void hz_leaf(const HzFace& f, float3 x0, float3 x1, float3 x2, float3& v, float& r,
+                                                 float& hb) {
+  const float3 q0 = x0 - f.v0, q1 = x1 - f.v0, q2 = x2 - f.v0, c = (q0 + q1 + q2) * (1.0f / 3.0f);
+  v = c - f.c;
+  r = hz_sqrt(fmaxf(dot3(q0 - c, q0 - c), fmaxf(dot3(q1 - c, q1 - c), dot3(q2 - c, q2 - c))));
+  hb = fmaxf(dot3(q0, f.n), fmaxf(dot3(q1, f.n), dot3(q2, f.n)));
+}
+// what a child's bound is widened by, for rounding: height and radius
+__host__ __device__ __forceinline__ float hz_slack(const HzFace& f, float3 v, float r) {
+  return 1e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + r + f.r);
+}
+// the finer bound of a triangle near f
+__host__ __device__ __forceinline__ HzCells hz_fine(const HzFace& f, const float* ln, float3 x0, float3 x1, float3 x2) {
+  constexpr HzLines LN = hz_lines();
+  const float3 x[3] = {x0, x1, x2};
+  float X[3], Y[3], h[3];
+  int sh[3];   // the vertex of f this vertex is, or -1
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    auto same = [&](float3 a) { return x[i].x == a.x && x[i].y == a.y && x[i].z == a.z; };
+    sh[i] = same(f.v0) ? 0 : same(f.v1) ? 1 : same(f.v2) ? 2 : -1;
+    float3 q = x[i] - f.v0;
+    X[i] = dot3(q, f.T); Y[i] = dot3(q, f.B);
+    h[i] = dot3(q, f.n) + 1e-6f * (fabsf(q.x) + fabsf(q.y) + fabsf(q.z));
+    if (sh[i] >= 0) h[i] = 0.0f;
+  }
+  float best = INFINITY;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const float mx = ln[k], my = ln[6 + k], mo = ln[12 + k];
+    float d[3], tn = 0.0f;
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      d[i] = mx * X[i] + my * Y[i] - mo - 5e-7f * (fabsf(X[i]) + fabsf(Y[i]) + 2.0f * f.r);   // less its rounding
+      // a vertex of f on the border line itself
+      bool on = k < 3 ? (sh[i] == k || sh[i] == (k == 2 ? 0 : k + 1)) : sh[i] == k - 3;
+      if (on) d[i] = 0.0f;
+      if (h[i] > 0.0f) {
+        ok &= d[i] > f.tiny;
+        tn = fmaxf(tn, h[i] / d[i]);
+      }
+    }
+    // where the triangle's edges cross height 0 the distance must not be negative
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (i != j && h[i] > 0.0f && !(h[j] > 0.0f)) {
+          float cr = d[j] * h[i] - d[i] * h[j];
+          ok &= (sh[j] >= 0 && d[j] == 0.0f) || cr > 1e-4f * d[i] * (h[i] - h[j]);
+        }
+    if (ok) best = fminf(best, tn);
+  }
+  const float sn = best < 1e18f ? fminf(best * rsqrtf(1.0f + best * best) * 1.00001f, 1.0f) : 1.0f;
+  const float3 e1 = f.v1 - f.v0, e2 = f.v2 - f.v0;
+  const float fx[2] = {dot3(e1, f.T), dot3(e2, f.T)}, fy[2] = {dot3(e1, f.B), dot3(e2, f.B)};
+  float blo[8], bhi[8], clo[4], chi[4];
+  // products with w = x - y over the triangle's and f's vertices
+  auto range = [&](float lx, float ly, float& lo, float& hi) {
+    float a0 = lx * X[0] + ly * Y[0], a1 = lx * X[1] + ly * Y[1], a2 = lx * X[2] + ly * Y[2];
+    float f1 = lx * fx[0] + ly * fy[0], f2 = lx * fx[1] + ly * fy[1];
+    lo = fminf(a0, fminf(a1, a2)) - fmaxf(0.0f, fmaxf(f1, f2));
+    hi = fmaxf(a0, fmaxf(a1, a2)) - fminf(0.0f, fminf(f1, f2));
+  };
+#pragma unroll
+  for (int k = 0; k < 8; ++k) range(LN.bx[k], LN.by[k], blo[k], bhi[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) range(LN.cx[k], LN.cy[k], clo[k], chi[k]);
+  return hz_cells(hz_sectors(blo, bhi, clo, chi, f.tiny), -1.0f, sn);
+}
+
 __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __restrict__ nodes,
                                                            const float4* __restrict__ tri, int nf, int n4,
                                                            const MeshStat* ms, const float4* __restrict__ N,
@@ -231,156 +403,35 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
                                                            int* err) {
   __shared__ int stack_[HZ_WARPS][HZ_STACK], cand_[HZ_WARPS][64];
   __shared__ float lines_[HZ_WARPS][18];   // f's border lines (mx, my, mo): the finer bound's alone, kept off the registers
-  constexpr HzLines LN = hz_lines();
   const unsigned ALL = 0xffffffffu;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   int *stack = stack_[warp], *cand = cand_[warp];
   const int li = blockIdx.x * HZ_WARPS + warp;
   if (li >= nf) return;
-  const float3 v0 = xyz(tri[3 * li]), v1 = xyz(tri[3 * li + 1]), v2 = xyz(tri[3 * li + 2]);
-  const float3 e1 = v1 - v0, e2 = v2 - v0;
-  const float3 m = cross3(e1, e2);
-  const float l1 = len3(e1), l2 = len3(e2), l3 = len3(v2 - v1), ml = len3(m);
   const float side = ms->winding < 0 ? -1.0f : 1.0f;
-  const float lmax = fmaxf(l1, fmaxf(l2, l3));
-  // a sliver's normal and borders are not known well enough: nothing is free on it
-  const bool bad = !(ml > 1e-3f * lmax * lmax) || !(l1 > 1e-3f * lmax);
-  unsigned M[4] = {0u, 0u, 0u, 0u};   // marked cells: sector 2 w in the low half of word w, 2 w + 1 in the high
+  HzFace f;
+  const bool bad = !hz_face(xyz(tri[3 * li]), xyz(tri[3 * li + 1]), xyz(tri[3 * li + 2]), side, f);
+  unsigned M[4] = {0u, 0u, 0u, 0u};
   if (!bad) {
-    const float3 n = m * (side / ml), T = e1 * (1.0f / l1), B = cross3(n, T);
-    const float3 cf = (v0 + v1 + v2) * (1.0f / 3.0f);
-    const float rf = fmaxf(len3(v0 - cf), fmaxf(len3(v1 - cf), len3(v2 - cf)));
-    {
-      // f in its plane: outward edge normals (f runs clockwise about n when side < 0) and their bisectors
-      float* ln = lines_[warp];
-      if (lane < 3) {
-        auto in2 = [&](int k) { float3 d = (k == 0 ? v0 : k == 1 ? v1 : v2) - cf; return make_float2(dot3(d, T), dot3(d, B)); };
-        const float2 p0 = in2(lane), p1 = in2(lane == 2 ? 0 : lane + 1), p2 = in2(lane == 0 ? 2 : lane - 1);
-        auto normal = [&](float2 a, float2 b) {
-          float dx = b.x - a.x, dy = b.y - a.y, il = side / sqrtf(dx * dx + dy * dy);
-          return make_float2(dy * il, -dx * il);
-        };
-        const float2 m0 = normal(p0, p1), m1 = normal(p2, p0);   // of the edges that start and end at vertex `lane`
-        ln[lane] = m0.x; ln[6 + lane] = m0.y;
-        ln[12 + lane] = fmaxf(m0.x * p0.x + m0.y * p0.y, m0.x * p1.x + m0.y * p1.y);
-        const float sx = m0.x + m1.x, sy = m0.y + m1.y, il = rsqrtf(fmaxf(sx * sx + sy * sy, 1e-12f));
-        ln[3 + lane] = sx * il; ln[9 + lane] = sy * il;
-        ln[15 + lane] = (sx * p0.x + sy * p0.y) * il;
-      }
-      __syncwarp();
-    }
-    const float tiny = 1e-6f * fminf(lmax, 1.0f);
+    if (lane < 3) hz_border(f, side, lane, lines_[warp]);
+    __syncwarp();
 
-    // the cells of elevations lo .. hi in the sectors sec
-    struct Cells { unsigned w[4]; };
-    auto cells = [&](unsigned sec, float lo, float hi) {
-      Cells c;
-      int b0 = max(0, (int)floorf(hz_band(lo) - 1e-3f)), b1 = min(15, (int)floorf(hz_band(hi) + 1e-3f));
-      unsigned m = b1 >= b0 ? (2u << b1) - (1u << b0) : 0u;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) c.w[w] = (sec >> (2 * w) & 1u ? m : 0u) | (sec >> (2 * w + 1) & 1u ? m << 16 : 0u);
-      return c;
-    };
-    auto fresh = [&](const Cells& c) {   // cells not marked yet
+    auto fresh = [&](const HzCells& c) {   // cells not marked yet
       return __popc(c.w[0] & ~M[0]) + __popc(c.w[1] & ~M[1]) + __popc(c.w[2] & ~M[2]) + __popc(c.w[3] & ~M[3]);
     };
-    auto mark = [&](bool on, const Cells& c) {   // the lanes' cells enter the warp's
+    auto mark = [&](bool on, const HzCells& c) {   // the lanes' cells enter the warp's
 #pragma unroll
       for (int w = 0; w < 4; ++w) M[w] |= __reduce_or_sync(ALL, on ? c.w[w] : 0u);
     };
-    // cells of points within r of cf + v, at most hb high; far: small enough to be taken so
-    auto sphere = [&](float3 v, float r, float hb, bool& far) {
-      const float d2 = dot3(v, v), vn = dot3(v, n), vx = dot3(v, T), vy = dot3(v, B);
-      unsigned sec = 0xffu;
-      float lo = -1.0f, hi = 1.0f;
-      far = false;
-      if (r * r < d2) {
-        const float iv = rsqrtf(d2), sv = vn * iv, sr = r * iv, cv = hz_sqrt(1.0f - sv * sv),
-                    cr = hz_sqrt(1.0f - sr * sr);
-        if (cv >= sr || sv < 0.0f) hi = sv * cr + cv * sr + 1e-4f;
-        if (cv >= sr || sv > 0.0f) lo = sv * cr - cv * sr - 1e-4f;
-        const float D = hz_sqrt(vx * vx + vy * vy) * 0.99999f - r;
-        if (D > 0.0f) {
-          hi = fminf(hi, hb * rsqrtf(D * D + hb * hb) * 1.00001f);
-          // azimuth of the centre and of its disk, in sectors: asin x <= x + (pi / 2 - 1) x^3 on [0, 1]
-          const float x = __fdividef(r, D + r), a = hz_atan2(vy, vx) * (4.0f / PI_F),
-                      w = (x + 0.5708f * x * x * x + HZ_WIDEN + 5e-3f) * (4.0f / PI_F);
-          const int s0 = (int)floorf(a - w), n = (int)floorf(a + w) - s0 + 1;
-          if (n < 8) {
-            const unsigned m = (1u << n) - 1u, t = (unsigned)s0 & 7u;
-            sec = (m << t | m >> (8u - t)) & 0xffu;
-          }
-        }
-        far = sr < HZ_FAR;
-      }
-      return cells(sec, lo, hi);
-    };
     // the finer bound of the triangles put aside
     auto fine = [&](int cnt) {
-      Cells cl = {{0u, 0u, 0u, 0u}};
-      bool on_ = false;
+      HzCells cl = {{0u, 0u, 0u, 0u}};
       if (lane < cnt) {
         const int lj = cand[lane];
-        float3 x[3] = {xyz(tri[3 * lj]), xyz(tri[3 * lj + 1]), xyz(tri[3 * lj + 2])};
-        float X[3], Y[3], h[3];
-        int sh[3];   // the vertex of f this vertex is, or -1
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          auto same = [&](float3 a) { return x[i].x == a.x && x[i].y == a.y && x[i].z == a.z; };
-          sh[i] = same(v0) ? 0 : same(v1) ? 1 : same(v2) ? 2 : -1;
-          float3 q = x[i] - cf;
-          X[i] = dot3(q, T); Y[i] = dot3(q, B);
-          h[i] = dot3(q, n) + 1e-6f * (fabsf(q.x) + fabsf(q.y) + fabsf(q.z));
-          if (sh[i] >= 0) h[i] = 0.0f;
-        }
-        float best = __int_as_float(0x7f800000);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          const float mx = lines_[warp][k], my = lines_[warp][6 + k], mo = lines_[warp][12 + k];
-          float d[3], tn = 0.0f;
-          bool ok = true;
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            d[i] = mx * X[i] + my * Y[i] - mo;
-            // a vertex of f on the border line itself
-            bool on = k < 3 ? (sh[i] == k || sh[i] == (k == 2 ? 0 : k + 1)) : sh[i] == k - 3;
-            if (on) d[i] = 0.0f;
-            if (h[i] > 0.0f) {
-              ok &= d[i] > tiny;
-              tn = fmaxf(tn, h[i] / d[i]);
-            }
-          }
-          // where the triangle's edges cross height 0 the distance must not be negative
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-              if (i != j && h[i] > 0.0f && !(h[j] > 0.0f)) {
-                float cr = d[j] * h[i] - d[i] * h[j];
-                ok &= (sh[j] >= 0 && d[j] == 0.0f) || cr > 1e-4f * d[i] * (h[i] - h[j]);
-              }
-          if (ok) best = fminf(best, tn);
-        }
-        const float sn = best < 1e18f ? fminf(best * rsqrtf(1.0f + best * best) * 1.00001f, 1.0f) : 1.0f;
-        const float fx[3] = {dot3(v0 - cf, T), dot3(v1 - cf, T), dot3(v2 - cf, T)},
-                    fy[3] = {dot3(v0 - cf, B), dot3(v1 - cf, B), dot3(v2 - cf, B)};
-        float blo[8], bhi[8], clo[4], chi[4];
-        // products with w = x - y over the triangle's and f's vertices
-        auto range = [&](float lx, float ly, float& lo, float& hi) {
-          float a0 = lx * X[0] + ly * Y[0], a1 = lx * X[1] + ly * Y[1], a2 = lx * X[2] + ly * Y[2];
-          float f0 = lx * fx[0] + ly * fy[0], f1 = lx * fx[1] + ly * fy[1], f2 = lx * fx[2] + ly * fy[2];
-          lo = fminf(a0, fminf(a1, a2)) - fmaxf(f0, fmaxf(f1, f2));
-          hi = fmaxf(a0, fmaxf(a1, a2)) - fminf(f0, fminf(f1, f2));
-        };
-#pragma unroll
-        for (int k = 0; k < 8; ++k) range(LN.bx[k], LN.by[k], blo[k], bhi[k]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) range(LN.cx[k], LN.cy[k], clo[k], chi[k]);
-        cl = cells(hz_sectors(blo, bhi, clo, chi, tiny), -1.0f, sn);
-        on_ = true;
+        cl = hz_fine(f, lines_[warp], xyz(tri[3 * lj]), xyz(tri[3 * lj + 1]), xyz(tri[3 * lj + 2]));
       }
-      mark(on_, cl);
+      mark(lane < cnt, cl);
     };
 
     // lane groups of four take a node's children each; the first rounds go up f's ancestors, nearest first (the
@@ -408,26 +459,23 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
       }
       // the child's sphere about its own centre and how high it reaches over f's plane
       float3 v = mk3(0, 0, 0);
-      float r = 0.0f, hb = -1.0f, mag = 0.0f;
+      float r = 0.0f, hb = -1.0f;
       if (ch >= 0) {
         HzNode q = hz_load(N, ch);
-        v = q.c - cf;
+        const float3 w = q.c - f.v0;
+        v = w - f.c;
         r = q.R;
-        hb = dot3(v, n) + hz_support(q, n);
+        hb = dot3(w, f.n) + hz_support(q, f.n);
       } else if (ch != (int)0x80000000 && (unsigned)~ch < (unsigned)nf) {
-        float3 x0 = xyz(tri[3 * ~ch]), x1 = xyz(tri[3 * ~ch + 1]), x2 = xyz(tri[3 * ~ch + 2]);
-        float3 c = (x0 + x1 + x2) * (1.0f / 3.0f);
-        v = c - cf;
-        r = hz_sqrt(fmaxf(dot3(x0 - c, x0 - c), fmaxf(dot3(x1 - c, x1 - c), dot3(x2 - c, x2 - c))));
-        hb = fmaxf(dot3(x0 - v0, n), fmaxf(dot3(x1 - v0, n), dot3(x2 - v0, n)));
+        hz_leaf(f, xyz(tri[3 * ~ch]), xyz(tri[3 * ~ch + 1]), xyz(tri[3 * ~ch + 2]), v, r, hb);
       }
-      mag = fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + r + rf;
-      hb += 1e-6f * mag;
+      const float slack = hz_slack(f, v, r);
+      hb += slack;
       bool open = false, put = false, on = false;
-      Cells cl = {{0u, 0u, 0u, 0u}};
+      HzCells cl = {{0u, 0u, 0u, 0u}};
       if (hb > 0.0f) {
         bool far;
-        cl = sphere(v, (r + rf) * 1.00001f + 1e-6f * mag, hb, far);
+        cl = hz_sphere(f, v, (r + f.r) * 1.00001f + slack, hb, far);
         const int fr = fresh(cl);
         on = fr > 0;
         open = fr > HZ_FEW && !far && ch >= 0;
@@ -459,8 +507,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
 }
 
 // The free directions of a path vertex p on the face (v0, v1, v2) with the marked cells w; n: its unit normal turned
-// toward the incoming ray, `front` when that is the side of its winding. Unusable (on = false) on the surface's
-// inner side, or where p lies too far off the face.
+// toward the incoming ray (the surface's outer side). Unusable (on = false) where p lies too far off the face.
 struct HzPoint {
   float3 T, B, n;
   uint4 w;
@@ -468,12 +515,10 @@ struct HzPoint {
   bool on;
 };
 
-__device__ __forceinline__ HzPoint hz_point(const MeshStat* ms, const uint4* cells, int leaf, float3 p, float3 v0,
-                                            float3 v1, float3 v2, float3 n, bool front) {
+__host__ __device__ __forceinline__ HzPoint hz_point(float eta, uint4 cells, float3 p, float3 v0, float3 v1, float3 v2,
+                                                     float3 n) {
   HzPoint z;
-  z.on = front == (ms->winding >= 0);
-  if (!z.on) return z;
-  z.w = __ldg(&cells[leaf]);
+  z.w = cells;
   float3 e1 = v1 - v0, e2 = v2 - v0, q = p - v0, m = cross3(e1, e2);
   z.n = n;
   z.T = e1 * rsqrtf(dot3(e1, e1));
@@ -484,30 +529,35 @@ __device__ __forceinline__ HzPoint hz_point(const MeshStat* ms, const uint4* cel
   float b1 = fmaxf(r1, 0.0f), b2 = fmaxf(r2, 0.0f);
   float sc = b1 + b2 > 1.0f ? 1.0f / (b1 + b2) : 1.0f;
   float3 e = q - (e1 * b1 + e2 * b2) * sc;
-  float en = dot3(e, n), rho = (len3(e) + ms->eta) * (1.0f / T_EPS);
+  float en = dot3(e, n), rho = (len3(e) + eta) * (1.0f / T_EPS);
   z.on = rho <= HZ_RHO;
   z.rho = rho;
   z.irho = 1.0f / (1.0f + rho);
-  z.lo = HZ_MARGIN + (fmaxf(-en, 0.0f) + ms->eta) * (1.0f / T_EPS);
-  z.hi = HZ_MARGIN + (fmaxf(en, 0.0f) + ms->eta) * (1.0f / T_EPS);
+  z.lo = HZ_MARGIN + (fmaxf(-en, 0.0f) + eta) * (1.0f / T_EPS);
+  z.hi = HZ_MARGIN + (fmaxf(en, 0.0f) + eta) * (1.0f / T_EPS);
   // least distance to an edge: least weight times least altitude
   const float3 e3 = e2 - e1;
   const float w = fminf(fminf(r1, r2), 1.0f - r1 - r2) *
                   sqrtf(dot3(m, m) / fmaxf(dot3(e1, e1), fmaxf(dot3(e2, e2), dot3(e3, e3))));
-  z.least = ms->eta / w;
+  z.least = rho * T_EPS / w;
   z.on = z.on && w > 0.0f;
   return z;
 }
 
 // True when a ray from the vertex along the unit direction d is known to hit nothing but its own face.
-__device__ __forceinline__ bool hz_free(const HzPoint& z, float3 d) {
+__host__ __device__ __forceinline__ bool hz_free(const HzPoint& z, float3 d) {
   if (!z.on) return false;
   float dn = dot3(d, z.n), lo = hz_band((dn - z.lo) * z.irho);
   if (!(lo >= 0.0f) || !(dn > z.least)) return false;
-  int b0 = min((int)lo, 15), b1 = 15;
-  if (z.rho < 0.25f) b1 = min((int)hz_band((dn + z.hi) * (1.0f + 1.34f * z.rho)), 15);   // / (1 - rho)
+  int b0 = (int)lo, b1 = 15;
+  b0 = b0 < 15 ? b0 : 15;
+  if (z.rho < 0.25f) {   // / (1 - rho)
+    const int top = (int)hz_band((dn + z.hi) * (1.0f + 1.34f * z.rho));
+    b1 = top < 15 ? top : 15;
+  }
   unsigned band = (2u << b1) - (1u << b0), w;
-  if (z.rho * z.rho > HZ_WIDEN * HZ_WIDEN * (1.0f - dn * dn)) {   // the azimuth is too uncertain
+  const float turn = z.rho + HZ_TILT;
+  if (turn * turn > HZ_SIN * HZ_SIN * (1.0f - dn * dn)) {   // the azimuth is too uncertain
     w = z.w.x | z.w.y | z.w.z | z.w.w;
     w |= w >> 16;
   } else {

@@ -1100,8 +1100,9 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
       float3 n = back ? -ng : ng;
       // shading normal: n, or interpolated; a direction counts only above both
       float3 ns = c.smooth ? shading_normal(c, f, p, v0, v1, v2, back ? -1.0f : 1.0f) : n;
-      HzPoint hz;
-      if (HZ) hz = hz_point(c.mstat, c.hz, h.x, p, v0, v1, v2, n, !back);
+      HzPoint hz;   // the face's free directions are those of the surface's outer side
+      hz.on = false;
+      if (HZ && back == (c.mstat->winding < 0)) hz = hz_point(c.mstat->eta, __ldg(&c.hz[h.x]), p, v0, v1, v2, n);
       int tex = texel_of(c, f, p, v0, v1, v2);
       Mat m = fetch_mat(c.P, tex);
       if (c.sig) sig_mix(hs, (uint32_t)f);
