@@ -10,6 +10,7 @@
 // whole library follows.
 #pragma once
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 namespace st {
@@ -120,6 +121,37 @@ __device__ __forceinline__ float3 cam_project_jt(const DevView& v, float3 X, flo
   float3 dpx = (v.right - v.fwd * (sx * v.kx)) * ((float)v.W * 0.5f / (z * v.kx));
   float3 dpy = (v.up - v.fwd * (sy * v.ky)) * (-(float)v.H * 0.5f / (z * v.ky));
   return dpx * nx + dpy * ny;
+}
+
+// ------------------------------------------------------------------ edge candidates
+// What a sample needs of its candidate: the screen segment's start and extent, the clipped parameter range, the
+// clipped length and the unit normal. Computed once per candidate with the lists (k_edge_compact), since thousands
+// of samples take the same one and this is most of a sample's arithmetic (a projection and a clip: six divisions).
+struct EdgeRec {
+  float2 sa, ext, ns;
+  float t0, dt, len;
+  int e;
+};
+// A record's 48 bytes; one that is not drawable holds no edge, and no sample is taken of it.
+__host__ __device__ __forceinline__ void edge_pack(bool drawable, const EdgeRec& r, float4* p) {
+  const int e = drawable ? r.e : -1;
+  float bits;
+  memcpy(&bits, &e, sizeof(bits));
+  p[0] = make_float4(0, 0, 0, 0);
+  p[1] = make_float4(0, 0, 0, bits);
+  p[2] = make_float4(0, 0, 0, 0);
+  if (!drawable) return;
+  p[0] = make_float4(r.sa.x, r.sa.y, r.ext.x, r.ext.y);
+  p[1] = make_float4(r.t0, r.dt, r.len, bits);
+  p[2] = make_float4(r.ns.x, r.ns.y, 0.0f, 0.0f);
+}
+__host__ __device__ __forceinline__ bool edge_unpack(float4 a, float4 b, float4 d, EdgeRec& r) {
+  memcpy(&r.e, &b.w, sizeof(r.e));
+  r.sa = make_float2(a.x, a.y);
+  r.ext = make_float2(a.z, a.w);
+  r.t0 = b.x; r.dt = b.y; r.len = b.z;
+  r.ns = make_float2(d.x, d.y);
+  return r.e >= 0;
 }
 
 // ------------------------------------------------------------------ watertight ray/triangle

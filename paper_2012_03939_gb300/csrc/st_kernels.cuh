@@ -214,15 +214,6 @@ struct EdgeSample {
   float2 S, ns;
 };
 
-// What a sample needs of its candidate: the screen segment's start and extent, the clipped parameter range, the
-// clipped length and the unit normal. Computed once per candidate with the lists (k_edge_compact), since thousands
-// of samples take the same one and this is most of a sample's arithmetic (a projection and a clip: six divisions).
-struct EdgeRec {
-  float2 sa, ext, ns;
-  float t0, dt, len;
-  int e;
-};
-
 __device__ __forceinline__ bool edge_record(const KCtx& c, const DevView& v, int e, EdgeRec& r) {
   float2 sb;
   float t1;
@@ -252,12 +243,7 @@ __device__ __forceinline__ EdgeSample edge_sample(const KCtx& c, int vi, const D
   EdgeRec r;
   if (i < c.edge_cap) {
     const float4* p = c.edge_rec + 3 * ((size_t)vi * c.edge_cap + i);
-    float4 a = __ldg(p), b = __ldg(p + 1), d = __ldg(p + 2);
-    r.sa = make_float2(a.x, a.y);
-    r.ext = make_float2(a.z, a.w);
-    r.t0 = b.x; r.dt = b.y; r.len = b.z;
-    r.e = __float_as_int(b.w);
-    r.ns = make_float2(d.x, d.y);
+    if (!edge_unpack(__ldg(p), __ldg(p + 1), __ldg(p + 2), r)) return s;
   } else if (!edge_record(c, v, c.edge_cand[(size_t)vi * c.n_edges + i], r)) {
     return s;
   }
@@ -336,12 +322,11 @@ __global__ void __launch_bounds__(EDGE_TILE) k_edge_compact(KCtx c) {
   c.edge_cand[(size_t)vi * c.n_edges + at] = e;
   if (REC && at < c.edge_cap) {
     const DevView& v = c.views[vi];
+    // The flag is another kernel's clip of the same segment, which may round differently where it only touches the
+    // image: every place of the list gets a record all the same.
     EdgeRec r;
-    if (!edge_record(c, v, e, r)) return;   // flagged, so it is drawable
-    float4* p = c.edge_rec + 3 * ((size_t)vi * c.edge_cap + at);
-    p[0] = make_float4(r.sa.x, r.sa.y, r.ext.x, r.ext.y);
-    p[1] = make_float4(r.t0, r.dt, r.len, __int_as_float(r.e));
-    p[2] = make_float4(r.ns.x, r.ns.y, 0.0f, 0.0f);
+    const bool drawable = edge_record(c, v, e, r);
+    edge_pack(drawable, r, c.edge_rec + 3 * ((size_t)vi * c.edge_cap + at));
   }
 }
 
