@@ -42,8 +42,8 @@
 // must also be steeper than (|e| + eta) / w, w the distance of p to f's nearest edge.
 // (Of 6 10^8 sampled free rays, half from within 10^-5 of an edge's length of it, one
 // had such a hit without this. With it: none of 3.4 10^9 over twelve meshes about the
-// origin, and of 7.7 10^9 rays from a face to one neighbour, coordinates up to 10^4 and
-// faces from 10^-3 to 5, no free one hit; with eta / w alone one did, at 10^3.)
+// origin, and of 10^10 rays past one neighbour, coordinates up to 10^4 and faces from
+// 10^-3 to 5, with and without fused products, no free one hit.)
 //
 // Measured on one GB300. k_horizon is bounded by instruction issue (55 % active, 16 to
 // 24 warps per SM, 15 of 32 lanes: nodes and triangles of a round take different
@@ -71,6 +71,7 @@ constexpr float HZ_RHO = 4.0f;        // largest rho for which the directions ar
 constexpr float HZ_MARGIN = 0.003f;   // constant part of the elevation margin (rounding of the frames)
 constexpr float HZ_FLOOR = 0.003f;    // sine of elevation below which nothing is free
 constexpr float HZ_LOW = 0.02f;       // upper end of the lowest band: what a gentle surface's neighbours reach
+constexpr float HZ_THIN = 1.0f / 256;   // twice the area over the longest edge squared up to which a triangle is a needle
 constexpr int HZ_FEW = 1;             // cells not marked yet up to which a node is taken by its sphere too
 constexpr float HZ_FAR = 0.2f;        // radius over distance of a node (or triangle) taken by its sphere
 constexpr int HZ_WARPS = 8;           // warps (faces) of a k_horizon block
@@ -323,13 +324,20 @@ __host__ __device__ __forceinline__ HzCells hz_sphere(const HzFace& f, float3 v,
   }
   return hz_cells(sec, lo, hi);
 }
-// a triangle's sphere about its own centre (v from f's) and how high it reaches over f's plane
-__host__ __device__ __forceinline__ void hz_leaf(const HzFace& f, float3 x0, float3 x1, float3 x2, float3& v, float& r,
+// A triangle's sphere about its own centre (v from f's) and how high it reaches over f's plane; true when it may have the
+// finer bound. A needle may not: the watertight test's depth on it is off by the rounding of its height over its length,
+// and from a vertex that it touches it may be reported past T_EPS in any direction. Near f its sphere marks every cell.
+__host__ __device__ __forceinline__ bool hz_leaf(const HzFace& f, float3 x0, float3 x1, float3 x2, float3& v, float& r,
                                                  float& hb) {
   const float3 q0 = x0 - f.v0, q1 = x1 - f.v0, q2 = x2 - f.v0, c = (q0 + q1 + q2) * (1.0f / 3.0f);
   v = c - f.c;
   r = hz_sqrt(fmaxf(dot3(q0 - c, q0 - c), fmaxf(dot3(q1 - c, q1 - c), dot3(q2 - c, q2 - c))));
   hb = fmaxf(dot3(q0, f.n), fmaxf(dot3(q1, f.n), dot3(q2, f.n)));
+  const float3 e1 = q1 - q0, e2 = q2 - q0, m = cross3(e1, e2), e3 = q2 - q1;
+  const float l2 = fmaxf(dot3(e1, e1), fmaxf(dot3(e2, e2), dot3(e3, e3)));
+  const bool thin = !(dot3(m, m) > HZ_THIN * HZ_THIN * l2 * l2);
+  if (thin) hb += HZ_THIN * (r + f.r);
+  return !thin;
 }
 // what a child's bound is widened by, for rounding: height and radius
 __host__ __device__ __forceinline__ float hz_slack(const HzFace& f, float3 v, float r) {
@@ -460,6 +468,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
       // the child's sphere about its own centre and how high it reaches over f's plane
       float3 v = mk3(0, 0, 0);
       float r = 0.0f, hb = -1.0f;
+      bool finer = false;
       if (ch >= 0) {
         HzNode q = hz_load(N, ch);
         const float3 w = q.c - f.v0;
@@ -467,7 +476,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
         r = q.R;
         hb = dot3(w, f.n) + hz_support(q, f.n);
       } else if (ch != (int)0x80000000 && (unsigned)~ch < (unsigned)nf) {
-        hz_leaf(f, xyz(tri[3 * ~ch]), xyz(tri[3 * ~ch + 1]), xyz(tri[3 * ~ch + 2]), v, r, hb);
+        finer = hz_leaf(f, xyz(tri[3 * ~ch]), xyz(tri[3 * ~ch + 1]), xyz(tri[3 * ~ch + 2]), v, r, hb);
       }
       const float slack = hz_slack(f, v, r);
       hb += slack;
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
         const int fr = fresh(cl);
         on = fr > 0;
         open = fr > HZ_FEW && !far && ch >= 0;
-        put = fr > HZ_FEW && !far && ch < 0;
+        put = fr > HZ_FEW && !far && finer;
       }
       const unsigned mo_ = __ballot_sync(ALL, open), mp = __ballot_sync(ALL, put);
       const int room = min(HZ_STACK - sp, HZ_OPEN - opened), at = __popc(mo_ & below), add = min(__popc(mo_), room);

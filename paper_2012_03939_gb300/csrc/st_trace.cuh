@@ -20,13 +20,13 @@ constexpr int ERR_INDEX = 8;  // a leaf or bin-list index outside its array (the
 
 struct TraceStats { int visits, tests; };
 
-__device__ __forceinline__ float3 safe_inv(float3 d) {
+__host__ __device__ __forceinline__ float3 safe_inv(float3 d) {
   auto inv1 = [](float x) { return fabsf(x) > 1e-30f ? 1.0f / x : copysignf(1e30f, x); };
   return mk3(inv1(d.x), inv1(d.y), inv1(d.z));
 }
 
 // slab test of box [lo, hi]; returns entry distance or +inf on a miss
-__device__ __forceinline__ float box_hit(float lx, float hx, float ly, float hy, float lz, float hz, float3 o,
+__host__ __device__ __forceinline__ float box_hit(float lx, float hx, float ly, float hy, float lz, float hz, float3 o,
                                          float3 inv, float tmax) {
   float tx0 = (lx - o.x) * inv.x, tx1 = (hx - o.x) * inv.x;
   float ty0 = (ly - o.y) * inv.y, ty1 = (hy - o.y) * inv.y;
@@ -35,7 +35,7 @@ __device__ __forceinline__ float box_hit(float lx, float hx, float ly, float hy,
   float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), tmax));
   // widen the far distance by 1 + 2*gamma(3) so rounding never culls a hit
   // (Ize, "Robust BVH Ray Traversal", JCGT 2013)
-  return tn <= tf * 1.00000036f ? tn : __int_as_float(0x7f800000);
+  return tn <= tf * 1.00000036f ? tn : INFINITY;
 }
 
 // ANY = stop at the first hit (shadow rays). nf = leaves (faces), nn = 4-wide

@@ -42,7 +42,7 @@ float3 narrow(D3 a) { return make_float3((float)a.x, (float)a.y, (float)a.z); }
 st::HzCells marks(const st::HzFace& f, const float* ln, const float3 (&x)[3]) {
   float3 v;
   float r, hb;
-  st::hz_leaf(f, x[0], x[1], x[2], v, r, hb);
+  const bool finer = st::hz_leaf(f, x[0], x[1], x[2], v, r, hb);
   const float slack = st::hz_slack(f, v, r);
   hb += slack;
   if (!(hb > 0.0f)) return {{0u, 0u, 0u, 0u}};
@@ -51,7 +51,7 @@ st::HzCells marks(const st::HzFace& f, const float* ln, const float3 (&x)[3]) {
   int marked = 0;
   for (unsigned w : c.w)
     for (; w; w &= w - 1) ++marked;
-  return marked > st::HZ_FEW && !far ? st::hz_fine(f, ln, x[0], x[1], x[2]) : c;
+  return marked > st::HZ_FEW && !far && finer ? st::hz_fine(f, ln, x[0], x[1], x[2]) : c;
 }
 
 double longest(const float3 (&a)[3]) {
@@ -61,6 +61,18 @@ double longest(const float3 (&a)[3]) {
     l = std::fmax(l, std::sqrt(dot(e, e)));
   }
   return l;
+}
+
+// what a traversal finds of the neighbour: its box, then the watertight test
+bool hit(float3 p, float3 d, const float3 (&x)[3]) {
+  const float3 inv = st::safe_inv(d);
+  auto lo = [](float a, float b, float c) { return fminf(a, fminf(b, c)); };
+  auto hi = [](float a, float b, float c) { return fmaxf(a, fmaxf(b, c)); };
+  if (st::box_hit(lo(x[0].x, x[1].x, x[2].x), hi(x[0].x, x[1].x, x[2].x), lo(x[0].y, x[1].y, x[2].y),
+                  hi(x[0].y, x[1].y, x[2].y), lo(x[0].z, x[1].z, x[2].z), hi(x[0].z, x[1].z, x[2].z), p, inv,
+                  INFINITY) == INFINITY)
+    return false;
+  return st::tri_test(st::ray_pre(p, d), x[0], x[1], x[2], INFINITY) > 0.0f;
 }
 
 }  // namespace
@@ -129,7 +141,7 @@ extern "C" long long hz_check(unsigned long long seed, long long pairs, int rays
       const st::HzPoint z = st::hz_point(eta, make_uint4(c.w[0], c.w[1], c.w[2], c.w[3]), p, f[0], f[1], f[2], n);
       if (!st::hz_free(z, d)) continue;
       ++out[1];
-      if (st::tri_test(st::ray_pre(p, d), x[0], x[1], x[2], INFINITY) > 0.0f) ++wrong;
+      if (hit(p, d, x)) ++wrong;
     }
   }
   return wrong;
