@@ -1389,8 +1389,7 @@ st_status st_scene_create(const st_scene_desc* d, void* stream, st_scene** out) 
   {
     const size_t m4 = (size_t)std::max(n - 1, 1);
     chk(dalloc(&s->parent4, m4)); chk(dalloc(&s->leaf_node4, (size_t)n));
-    // one record more than there are nodes: the hierarchy's build takes hz and hz_nodes as scratch
-    chk(dalloc(&s->hz, (size_t)n)); chk(dalloc(&s->hz_nodes, 3 * m4 + 1)); chk(dalloc(&s->hz_done, m4));
+    chk(dalloc(&s->hz, (size_t)n)); chk(dalloc(&s->hz_nodes, ploc_scratch(n).records)); chk(dalloc(&s->hz_done, m4));
   }
   {
     // edge hierarchy: at most 2^14 leaf blocks of at least 4 edges

@@ -477,12 +477,12 @@ cudaError_t bvh_build_ploc(st_scene* s, cudaStream_t stream) {
   cudaError_t e = morton_order(s, stream);
   if (e != cudaSuccess || n < 2) return e != cudaSuccess ? e : boxes(s, stream);
   // Scratch for the rounds: two cluster arrays (box, id), scans, neighbours. All of it is the scene's own memory whose
-  // content the build makes stale or has used already: the free directions (4 n - 2 float4), the collapse's queues (4 n
+  // content the build makes stale or has used already: the free directions (4 n float4), the collapse's queues (4 n
   // ints) and the sort's keys and second buffers (n ints each). Allocated per call it cost an allocation, a
   // synchronisation and a release.
-  float4* hzn = s->hz_nodes;
-  float4* lo[2] = {reinterpret_cast<float4*>(s->hz), hzn + n};   // n, n - 1
-  float4* hi[2] = {hzn, hzn + 2 * (size_t)n - 1};                // n, n - 1
+  const PlocScratch at = ploc_scratch(n);
+  float4* lo[2] = {reinterpret_cast<float4*>(s->hz), s->hz_nodes + at.lo1};
+  float4* hi[2] = {s->hz_nodes + at.hi0, s->hz_nodes + at.hi1};
   int2* scan = reinterpret_cast<int2*>(s->q4);
   int2* part = scan + n;   // of n / SCAN2_BLOCK blocks and the total: at most n
   int* cid[2] = {reinterpret_cast<int*>(s->keys2), s->ids2};

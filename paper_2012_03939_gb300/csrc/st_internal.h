@@ -238,4 +238,10 @@ cudaError_t trace_closest(st_scene* s, const float* rays, int n, int exclude, in
 void set_error(const std::string& msg);
 bool fault_now(int site);   // host-side fault injection: true when this event at `site` is to fail
 int sort_blocks_for(int n);
+
+// hz_nodes: the free directions' node records (3 of each of up to n - 1 nodes), and between two builds of them the scratch
+// of the hierarchy's clustering: its second and third arrays of n cluster boxes each (a round that merges nothing, on
+// boxes that are not finite, writes all n before the host reads that it did).
+struct PlocScratch { size_t lo1, hi0, hi1, records; };   // offsets and size, in float4
+constexpr PlocScratch ploc_scratch(size_t n) { return PlocScratch{n, 0, 2 * n, 3 * n}; }
 }  // namespace st
