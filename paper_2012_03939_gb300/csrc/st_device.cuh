@@ -201,6 +201,32 @@ __host__ __device__ __forceinline__ float tri_test(const RayPre& r, float3 p0, f
   return (t > T_EPS && t < tmax) ? t : -1.0f;
 }
 
+// ------------------------------------------------------------------ rounding as written
+// What shading computes with: every product and sum in these helpers, and in the functions below that use them, is rounded
+// as written. The compiler may fuse a product into either side of a sum and picks from kernel to kernel; shading's two
+// variants (st_kernels.cuh) take the same decisions and add the same terms, and have to agree bitwise. The orders are those
+// it had picked there, so that paths take the decisions that they took (dot_x_rn where it began with the x products).
+__device__ __forceinline__ float dot_rn(float3 a, float3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float dot_x_rn(float3 a, float3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
+__device__ __forceinline__ float3 cross_rn(float3 a, float3 b) {
+  return mk3(__fmaf_rn(a.y, b.z, -__fmul_rn(a.z, b.y)), __fmaf_rn(a.z, b.x, -__fmul_rn(a.x, b.z)),
+             __fmaf_rn(a.x, b.y, -__fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float3 norm_rn(float3 a) { float l = sqrtf(dot_rn(a, a)); return mk3(a.x / l, a.y / l, a.z / l); }
+__device__ __forceinline__ float3 add_rn(float3 a, float3 b) { return mk3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z)); }
+// a s + b
+__device__ __forceinline__ float3 mad_rn(float3 a, float s, float3 b) {
+  return mk3(__fmaf_rn(a.x, s, b.x), __fmaf_rn(a.y, s, b.y), __fmaf_rn(a.z, s, b.z));
+}
+// a s + b t + c u
+__device__ __forceinline__ float3 mix_rn(float3 a, float s, float3 b, float t, float3 c, float u) {
+  return mad_rn(c, u, mad_rn(a, s, mk3(__fmul_rn(b.x, t), __fmul_rn(b.y, t), __fmul_rn(b.z, t))));
+}
+
 // ------------------------------------------------------------------ environment
 struct DevEnv {
   int w, h;                 // 0 = no environment
@@ -210,13 +236,13 @@ struct DevEnv {
 };
 
 __device__ __forceinline__ int env_texel(const DevEnv& e, float3 d, float& sin_t) {
-  float phi = atan2f(d.x, -d.z) + PI_F;
+  float phi = __fadd_rn(atan2f(d.x, -d.z), PI_F);
   int col = (int)(phi * (1.0f / (2.0f * PI_F)) * (float)e.w);
   col = min(max(col, 0), e.w - 1);
   float th = acosf(fminf(fmaxf(d.y, -1.0f), 1.0f));
   int row = (int)(th * (1.0f / PI_F) * (float)e.h);
   row = min(max(row, 0), e.h - 1);
-  sin_t = sqrtf(fmaxf(0.0f, 1.0f - d.y * d.y));
+  sin_t = sqrtf(fmaxf(0.0f, __fmaf_rn(-d.y, d.y, 1.0f)));
   return row * e.w + col;
 }
 
@@ -238,8 +264,8 @@ struct Mat { float kd[3]; float ks[3]; float alpha; };
 
 // specular lobe probability: mean ks over mean ks + mean kd, clamped
 __device__ __forceinline__ float lobe_prob(const Mat& m) {
-  float ks = (m.ks[0] + m.ks[1] + m.ks[2]) * (1.0f / 3.0f);
-  float den = ks + (m.kd[0] + m.kd[1] + m.kd[2]) * (1.0f / 3.0f);
+  float ks = __fmul_rn(__fadd_rn(__fadd_rn(m.ks[0], m.ks[1]), m.ks[2]), 1.0f / 3.0f);
+  float den = __fmaf_rn(__fadd_rn(__fadd_rn(m.kd[0], m.kd[1]), m.kd[2]), 1.0f / 3.0f, ks);
   if (!(den > 0.0f)) return 0.5f;
   return fminf(fmaxf(ks / den, 0.05f), 0.95f);
 }
@@ -319,12 +345,7 @@ __device__ __forceinline__ float3 brdf_cos(int brdf, int fr, const Mat& m, float
              m.kd[2] * kdc + (m.ks[2] + (1.0f - m.ks[2]) * x5) * spec);
 }
 
-// brdf_cos with every product and sum rounded as written. The compiler fuses a product into either side of a sum and
-// picks differently from kernel to kernel (with the register limit, too); shading's variants add the same terms and
-// have to agree bitwise.
-__device__ __forceinline__ float dot_rn(float3 a, float3 b) {
-  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
-}
+// brdf_cos with every product and sum rounded as written.
 __device__ __forceinline__ float D_rn(int brdf, float c, float a) {
   const float a2 = __fmul_rn(a, a), c2 = __fmul_rn(c, c);
   if (brdf == 0) {
@@ -347,18 +368,18 @@ __device__ __forceinline__ float G1_rn(int brdf, float c, float a) {
   return 2.0f / __fadd_rn(__fadd_rn(1.0f, erff(x)), e / __fmul_rn(x, 1.7724538509055160f));
 }
 __device__ __forceinline__ float3 brdf_cos_rn(int brdf, int fr, const Mat& m, float3 n, float3 wi, float3 wo) {
-  const float ci = dot_rn(n, wi), co = dot_rn(n, wo);
+  const float ci = dot_x_rn(n, wi), co = dot_x_rn(n, wo);
   if (!(ci > 0.0f) || !(co > 0.0f)) return mk3(0, 0, 0);
-  float3 h = mk3(__fadd_rn(wi.x, wo.x), __fadd_rn(wi.y, wo.y), __fadd_rn(wi.z, wo.z));
-  const float hl = sqrtf(dot_rn(h, h));
+  float3 h = add_rn(wi, wo);
+  const float hl = sqrtf(dot_x_rn(h, h));
   h = mk3(h.x / hl, h.y / hl, h.z / hl);
   bool cl;
   const float a = clamp_alpha(m.alpha, cl);
-  const float spec = __fmul_rn(__fmul_rn(D_rn(brdf, dot_rn(n, h), a), G1_rn(brdf, ci, a)), G1_rn(brdf, co, a)) /
+  const float spec = __fmul_rn(__fmul_rn(D_rn(brdf, dot_x_rn(n, h), a), G1_rn(brdf, ci, a)), G1_rn(brdf, co, a)) /
                      __fmul_rn(4.0f, co);
   float x5 = 0.0f;
   if (fr) {
-    const float x = __fsub_rn(1.0f, dot_rn(wi, h)), x2 = __fmul_rn(x, x);
+    const float x = __fsub_rn(1.0f, dot_x_rn(wi, h)), x2 = __fmul_rn(x, x);
     x5 = __fmul_rn(__fmul_rn(x2, x2), x);
   }
   const float kdc = __fmul_rn(ci, 1.0f / PI_F);
@@ -370,14 +391,15 @@ __device__ __forceinline__ float3 brdf_cos_rn(int brdf, int fr, const Mat& m, fl
 
 // One-sample lobe-mixture pdf (solid angle) of direction wi.
 __device__ __forceinline__ float brdf_pdf(int brdf, const Mat& m, float3 n, float3 wi, float3 wo) {
-  float ci = dot3(n, wi), co = dot3(n, wo);
+  float ci = dot_rn(n, wi), co = dot_rn(n, wo);
   if (!(ci > 0.0f) || !(co > 0.0f)) return 0.0f;
-  float3 h = norm3(wi + wo);
-  float ch = dot3(n, h), woh = fabsf(dot3(wo, h));
+  float3 h = norm_rn(add_rn(wi, wo));
+  float ch = dot_rn(n, h), woh = fabsf(dot_x_rn(wo, h));
   bool cl;
   float a = clamp_alpha(m.alpha, cl);
   float ps = lobe_prob(m);
-  return (1.0f - ps) * ci * (1.0f / PI_F) + ps * D_eval(brdf, ch, a) * ch / (4.0f * woh);
+  float spec = __fmul_rn(__fmul_rn(ps, D_rn(brdf, ch, a)), ch) / __fmul_rn(4.0f, woh);
+  return __fmaf_rn(__fmul_rn(__fsub_rn(1.0f, ps), ci), 1.0f / PI_F, spec);
 }
 
 // Orthonormal frame around n: t = (h x n)/|h x n|, b = n x t, helper axis h =
@@ -386,14 +408,14 @@ __device__ __forceinline__ float brdf_pdf(int brdf, const Mat& m, float3 n, floa
 // on a coordinate plane (symmetric meshes) get the same frame at any
 // precision; the lobes are isotropic, so the frame changes no density.
 __device__ __forceinline__ void onb(float3 n, float3& t, float3& b) {
-  float3 c = cross3(mk3(0.4375f, 0.5625f, 0.6875f), n);
-  float l2 = dot3(c, c);
+  float3 c = cross_rn(mk3(0.4375f, 0.5625f, 0.6875f), n);
+  float l2 = dot_rn(c, c);
   if (!(l2 > 1e-12f)) {
-    c = cross3(mk3(0.6875f, -0.4375f, 0.5625f), n);
-    l2 = dot3(c, c);
+    c = cross_rn(mk3(0.6875f, -0.4375f, 0.5625f), n);
+    l2 = dot_rn(c, c);
   }
   t = c * rsqrtf(l2);
-  b = cross3(n, t);
+  b = cross_rn(n, t);
 }
 
 // Returns the mixture pdf of the sampled direction wi; 0 = no valid sample.
@@ -405,30 +427,30 @@ __device__ __forceinline__ float brdf_sample(int brdf, const Mat& m, float3 n, f
   if (ul < ps) {
     bool cl;
     float a = clamp_alpha(m.alpha, cl);
-    float a2 = a * a;
-    float tan2 = brdf == 0 ? a2 * u1 / (1.0f - u1) : -a2 * logf(1.0f - u1);
-    float ch = rsqrtf(1.0f + tan2);
-    float sh = sqrtf(fmaxf(0.0f, 1.0f - ch * ch));
+    float a2 = __fmul_rn(a, a), r1 = __fsub_rn(1.0f, u1);
+    float sec2 = brdf == 0 ? __fadd_rn(1.0f, __fmul_rn(a2, u1) / r1) : __fadd_rn(1.0f, __fmul_rn(-a2, logf(r1)));   // of the half vector
+    float ch = rsqrtf(sec2);
+    float sh = sqrtf(fmaxf(0.0f, __fmaf_rn(-ch, ch, 1.0f)));
     float sp, cp;
     sincosf(2.0f * PI_F * u2, &sp, &cp);
-    float3 h = t * (sh * cp) + b * (sh * sp) + n * ch;
-    wi = h * (2.0f * dot3(wo, h)) - wo;
+    float3 h = mix_rn(t, __fmul_rn(sh, cp), b, __fmul_rn(sh, sp), n, ch);
+    wi = mad_rn(h, 2.0f * dot_x_rn(wo, h), -wo);
   } else {
     // concentric square-to-disk map (Shirley and Chiu 1997), then project up
-    float a = 2.0f * u1 - 1.0f, c = 2.0f * u2 - 1.0f;
+    float a = __fmaf_rn(2.0f, u1, -1.0f), c = __fmaf_rn(2.0f, u2, -1.0f);
     float x = 0.0f, y = 0.0f;
     if (a != 0.0f || c != 0.0f) {
       float r, ph;
       if (fabsf(a) > fabsf(c)) { r = a; ph = (PI_F * 0.25f) * (c / a); }
-      else { r = c; ph = PI_F * 0.5f - (PI_F * 0.25f) * (a / c); }
+      else { r = c; ph = __fmaf_rn(-(PI_F * 0.25f), a / c, PI_F * 0.5f); }
       float sp, cp;
       sincosf(ph, &sp, &cp);
-      x = r * cp; y = r * sp;
+      x = __fmul_rn(r, cp); y = __fmul_rn(r, sp);
     }
-    float z = sqrtf(fmaxf(0.0f, 1.0f - x * x - y * y));
-    wi = t * x + b * y + n * z;
+    float z = sqrtf(fmaxf(0.0f, __fmaf_rn(-y, y, __fmaf_rn(-x, x, 1.0f))));
+    wi = mix_rn(t, x, b, y, n, z);
   }
-  if (!(dot3(n, wi) > 0.0f)) return 0.0f;
+  if (!(dot_rn(n, wi) > 0.0f)) return 0.0f;
   return brdf_pdf(brdf, m, n, wi, wo);
 }
 

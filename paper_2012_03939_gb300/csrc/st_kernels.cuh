@@ -146,9 +146,9 @@ __device__ __forceinline__ int lights_of(const KCtx& c, int vi) {
 __device__ __forceinline__ int texel_of(const KCtx& c, int f, float3 p, float3 v0, float3 v1, float3 v2) {
   if (c.res == 0) return f;
   float3 e1 = v1 - v0, e2 = v2 - v0, q = p - v0;
-  float3 m = cross3(e1, e2);
-  float im = 1.0f / dot3(m, m);
-  float alpha = dot3(cross3(q, e2), m) * im, beta = dot3(cross3(e1, q), m) * im;
+  float3 m = cross_rn(e1, e2);
+  float im = 1.0f / dot_rn(m, m);
+  float alpha = dot_rn(cross_rn(q, e2), m) * im, beta = dot_rn(cross_rn(e1, q), m) * im;
   int r = c.res;
   int i = min(max((int)floorf((float)r * alpha), 0), r);
   int j = min(max((int)floorf((float)r * beta), 0), r - i);
@@ -162,11 +162,11 @@ __device__ __forceinline__ int texel_of(const KCtx& c, int f, float3 p, float3 v
 __device__ __forceinline__ float3 shading_normal(const KCtx& c, int f, float3 p, float3 v0, float3 v1, float3 v2,
                                                  float sgn) {
   float3 e1 = v1 - v0, e2 = v2 - v0, q = p - v0;
-  float3 m = cross3(e1, e2);
-  float mm = dot3(m, m);
-  float b1 = dot3(cross3(q, e2), m) / mm, b2 = dot3(cross3(e1, q), m) / mm;
+  float3 m = cross_rn(e1, e2);
+  float mm = dot_rn(m, m);
+  float b1 = dot_rn(cross_rn(q, e2), m) / mm, b2 = dot_rn(cross_rn(e1, q), m) / mm;
   float3 n0 = xyz(c.vn[c.F[3 * f]]), n1 = xyz(c.vn[c.F[3 * f + 1]]), n2 = xyz(c.vn[c.F[3 * f + 2]]);
-  return norm3(n0 * (1.0f - b1 - b2) + n1 * b1 + n2 * b2) * sgn;
+  return norm_rn(mix_rn(n0, __fsub_rn(__fsub_rn(1.0f, b1), b2), n1, b1, n2, b2)) * sgn;
 }
 
 // ------------------------------------------------------------------ edges
@@ -1040,7 +1040,7 @@ constexpr float SH_NONE = 0.0f, SH_TRACE = 1.0f, SH_FREE = 2.0f;
 // are built, every ray is traced (87 registers against 116).
 // Waits on loads with few warps (a third of the issue slots used at two blocks of 256 per SM), so it is held to seven
 // (without free directions six) blocks of 128: an iteration on 200k faces and 64 views 34.3 -> 31.9 ms, on 5120 faces
-// 3.91 -> 3.63, three planes 0.886 either way. What both variants add to a pixel is rounded as written (brdf_cos_rn).
+// 3.91 -> 3.63, three planes 0.886 either way. What both variants decide by and add to a pixel is rounded as written.
 constexpr int SHADE_BLOCK = 128;
 template <bool HZ>
 __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b, int first) {
@@ -1079,9 +1079,11 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
       float t = __int_as_float(h.y);
       float3 p = mk3(__fmaf_rn(dir.x, t, org.x), __fmaf_rn(dir.y, t, org.y), __fmaf_rn(dir.z, t, org.z));
       float3 v0 = xyz(ta), v1 = xyz(tb), v2 = xyz(tc);
-      float3 ng = norm3(cross3(v1 - v0, v2 - v0));
+      float3 ng = cross_rn(v1 - v0, v2 - v0);
+      const float nl = sqrtf(dot_rn(ng, ng));
+      ng = mk3(ng.x / nl, ng.y / nl, ng.z / nl);
       float3 wo = -dir;
-      const bool back = dot3(ng, wo) < 0.0f;
+      const bool back = dot_rn(ng, wo) < 0.0f;
       float3 n = back ? -ng : ng;
       // shading normal: n, or interpolated; a direction counts only above both
       float3 ns = c.smooth ? shading_normal(c, f, p, v0, v1, v2, back ? -1.0f : 1.0f) : n;
@@ -1101,14 +1103,14 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
       int sent = 0, open = 0;
       const int nlp = lights_of(c, vi);
       auto lit = [&](float3 wi, float dist) {
-        return dot3(n, wi) > 0.0f && dist > 2.0f * T_EPS && (!c.smooth || dot3(ns, wi) > 0.0f);
+        return dot_rn(n, wi) > 0.0f && dist > 2.0f * T_EPS && (!c.smooth || dot_rn(ns, wi) > 0.0f);
       };
       if (HZ)
         for (int j = 0; j < nlp; ++j) {
           float4 lp, li;
           point_light(c, vi, j, lp, li);
           float3 dv = xyz(lp) - p;
-          float dist = sqrtf(dot_rn(dv, dv));
+          float dist = sqrtf(dot_x_rn(dv, dv));
           float3 wi = dv * (1.0f / dist);
           if (lit(wi, dist)) {
             sent |= 1 << j;
@@ -1128,7 +1130,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
         sincosf(PI_F * vq, &esth, &cth);
         sincosf(2.0f * PI_F * uu, &sph, &cph);
         ewi = mk3(-esth * sph, cth, esth * cph);
-        if (esth > 0.0f && dot3(n, ewi) > 0.0f && (!c.smooth || dot3(ns, ewi) > 0.0f)) {
+        if (esth > 0.0f && dot_rn(n, ewi) > 0.0f && (!c.smooth || dot_rn(ns, ewi) > 0.0f)) {
           sent |= ENV_VIS;
           if (HZ && hz_free(hz, ewi)) open |= ENV_VIS;
         }
@@ -1140,7 +1142,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
         float4 lp = make_float4(0, 0, 1, 0), li = make_float4(0, 0, 0, 0);
         if (j < nlp) point_light(c, vi, j, lp, li);
         float3 dv = xyz(lp) - p;
-        float dist = sqrtf(dot_rn(dv, dv));
+        float dist = sqrtf(dot_x_rn(dv, dv));
         float3 wi = dv * (1.0f / dist);
         const bool valid = HZ ? (sent >> j & 1) != 0 : j < nlp && lit(wi, dist);
         float3 cc = mk3(0, 0, 0);
@@ -1190,7 +1192,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b
       if (vb < c.B - 1) {
         U4 u = philox((uint32_t)ct.x, (uint32_t)ct.y, (uint32_t)(vb << 4) | 2u, (uint32_t)ct.z, key.k0, key.k1);
         pdf = brdf_sample(c.brdf, m, ns, wo, unif(u.x), unif(u.y), unif(u.z), wi);
-        if (c.smooth && pdf > 0.0f && !(dot3(n, wi) > 0.0f)) pdf = 0.0f;   // below the face
+        if (c.smooth && pdf > 0.0f && !(dot_rn(n, wi) > 0.0f)) pdf = 0.0f;   // below the face
         if (c.sig) sig_mix(hs, (unif(u.x) < lobe_prob(m) ? 1u : 0u) | (pdf > 0.0f ? 2u : 0u));
         if (pdf > 0.0f) {
           float3 Qv = brdf_cos_rn(c.brdf, c.fresnel, m, ns, wi, wo);
