@@ -61,9 +61,11 @@ bool fault_now(int site) {
 namespace {
 
 constexpr int DEFAULT_CHUNK = 1 << 22;
-// Candidates per view whose screen records are kept (48 bytes each); the samples of later ones project their edge
-// themselves. A silhouette of the 1M-face mesh has some ten thousand edges.
+// Candidates per view whose screen records are kept (48 bytes each), and bytes of them in all views; the samples of later
+// candidates project their edge themselves. A silhouette of the 1M-face mesh has some ten thousand edges, and 64 views
+// of 2^15 records take 100 MB; a call of thousands of views keeps fewer of each.
 constexpr int EDGE_RECORDS = 1 << 15;
+constexpr long long EDGE_RECORD_BYTES = 256LL << 20;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
 // Whether a call uses the faces' free directions (k_horizon). A face costs 8 (smooth) to 17 ns (rough) to build; of the
@@ -424,6 +426,24 @@ st_status ensure_engine(st_scene* s, int Q, int B, int NS, bool records, bool se
   return r;
 }
 
+void free_edge_records(st_scene* s) {
+  dfree(s->edge_rec);
+  s->edge_cap = s->edge_rec_views = 0;
+}
+
+// The candidates' screen records of n_views views, as many as the limits and the memory allow. The call runs without them
+// too, so they are asked for after everything that it needs.
+void ensure_edge_records(st_scene* s, int n_views) {
+  if (n_views <= s->edge_rec_views) return;
+  cudaDeviceSynchronize();
+  drop_graphs(s);
+  free_edge_records(s);
+  const long long cap = std::min<long long>({s->n_edges, EDGE_RECORDS, EDGE_RECORD_BYTES / (48LL * n_views)});
+  if (cap > 0 && dalloc(&s->edge_rec, 3 * (size_t)n_views * cap) == cudaSuccess) s->edge_cap = (int)cap;
+  cudaGetLastError();
+  s->edge_rec_views = n_views;
+}
+
 st_status ensure_tables(st_scene* s, int n_views, int n_segs, bool edges) {
   int need = std::max(n_views, n_segs);
   if (need > s->view_cap) {
@@ -447,16 +467,13 @@ st_status ensure_tables(st_scene* s, int n_views, int n_segs, bool edges) {
     dfree(s->edge_flag);
     dfree(s->edge_cand);
     dfree(s->edge_ncand);
-    dfree(s->edge_rec);
+    free_edge_records(s);
     size_t n = (size_t)n_views * std::max(s->n_edges, 1);
-    s->edge_cap = std::min(s->n_edges, EDGE_RECORDS);
     if (dalloc(&s->edge_flag, (size_t)n_views * edge_flag_ints(s->n_edges)) != cudaSuccess ||
-        dalloc(&s->edge_cand, n) != cudaSuccess || dalloc(&s->edge_ncand, (size_t)n_views) != cudaSuccess ||
-        dalloc(&s->edge_rec, 3 * (size_t)n_views * s->edge_cap) != cudaSuccess) {
+        dalloc(&s->edge_cand, n) != cudaSuccess || dalloc(&s->edge_ncand, (size_t)n_views) != cudaSuccess) {
       dfree(s->edge_flag);
       dfree(s->edge_cand);
       dfree(s->edge_ncand);
-      dfree(s->edge_rec);
       s->edge_cap_views = 0;
       cudaGetLastError();
       return fail(ST_ERR_OOM, "edge tables");
@@ -1155,6 +1172,7 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
   bool want_two = p.o.mode == ST_MODE_BATCHED && !timing_call && chunk_count(p, Q) >= 2;
   r = ensure_engine(s, Q, p.B, NS, p.kind == 1, p.sec, p.shadow, want_two ? chunk_count(p, Q) : 1);
   if (r != ST_OK) return r;
+  if (p.edges) ensure_edge_records(s, (int)p.views.size());
   if (want_two) {
     // events for the fork, every chunk's resolve and the join, made before any capture
     long long need = chunk_count(p, Q) + 2 * OVERLAP_ENGINES;

@@ -148,7 +148,8 @@ struct st_scene {
   int* edge_cand = nullptr;      // [views * E]
   int* edge_ncand = nullptr;     // [views]
   float4* edge_rec = nullptr;    // [views * edge_cap * 3] screen records of the candidates
-  int edge_cap = 0;
+  int edge_cap = 0;              // records per view; 0: none
+  int edge_rec_views = 0;        // views they were asked for
   int edge_cap_views = 0;
   int* sh_flag = nullptr;        // [pairs * edge_flag_ints(E)] light-silhouette flags per (view, light)
   int* sh_cand = nullptr;        // [pairs * E] their ordered compaction
