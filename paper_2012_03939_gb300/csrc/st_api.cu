@@ -372,10 +372,13 @@ void drop_graphs(st_scene* s) {
   s->graphs.clear();
 }
 
+bool engine_fits(const Engine& e, int Q, int B, int NS, bool records, bool sec, bool shadow) {
+  return e.Q >= Q && e.NS >= NS && (!records || (e.records && e.B >= B)) &&
+         (!sec || e.sec_cap >= (long long)e.B * e.Q) && (!shadow || e.shadow);
+}
+
 st_status grow_engine(st_scene* s, Engine& e, int Q, int B, int NS, bool records, bool sec, bool shadow) {
-  if (e.Q >= Q && e.NS >= NS && (!records || (e.records && e.B >= B)) &&
-      (!sec || e.sec_cap >= (long long)e.B * e.Q) && (!shadow || e.shadow))
-    return ST_OK;
+  if (engine_fits(e, Q, B, NS, records, sec, shadow)) return ST_OK;
   // grow: keep the larger of old and new sizes so alternating calls do not thrash
   int nQ = std::max(Q, e.Q), nNS = std::max(NS, e.NS), nB = std::max(B, e.B);
   bool nrec = records || e.records;
@@ -414,16 +417,45 @@ st_status grow_engine(st_scene* s, Engine& e, int Q, int B, int NS, bool records
   return ST_OK;
 }
 
+// Does without the engines from number k on (1 = the second): their buffers are free again. False if there were none.
+bool drop_engines(st_scene* s, int k) {
+  bool any = false;
+  for (int i = k; i < OVERLAP_ENGINES; ++i) any = any || s->eng2[i - 1].Q > 0;
+  s->max_engines = std::min(s->max_engines, k);
+  if (!any) return false;
+  cudaDeviceSynchronize();
+  drop_graphs(s);
+  for (int i = k; i < OVERLAP_ENGINES; ++i) free_engine(s->eng2[i - 1]);
+  return true;
+}
+
 // The call's wavefront buffers: one engine, or up to OVERLAP_ENGINES when consecutive chunks are to overlap on their
-// streams (see enqueue_body). Engines past OVERLAP_REQUIRED that do not fit are done without, in later calls too.
+// streams (see enqueue_body). Engines past OVERLAP_REQUIRED are optional: each takes at most a quarter of the memory that is
+// free, so that the caller's own allocations keep most of it, and what does not fit is done without until the first
+// engine grows again.
 st_status ensure_engine(st_scene* s, int Q, int B, int NS, bool records, bool sec, bool shadow, long long chunks) {
+  const long long had = s->eng.bytes;
   st_status r = grow_engine(s, s->eng, Q, B, NS, records, sec, shadow);
-  for (int k = 1; r == ST_OK && k < std::min<long long>(chunks, s->max_engines); ++k) {
-    st_status x = grow_engine(s, s->eng2[k - 1], Q, B, NS, records, sec, shadow);
-    if (x != ST_OK && k < OVERLAP_REQUIRED) r = x;
-    else if (x != ST_OK) s->max_engines = k;
+  if (r != ST_OK) return r;
+  if (s->eng.bytes != had) s->max_engines = OVERLAP_ENGINES;
+  for (int k = 1; k < std::min<long long>(chunks, s->max_engines); ++k) {
+    Engine& e = s->eng2[k - 1];
+    if (k < OVERLAP_REQUIRED) {
+      r = grow_engine(s, e, Q, B, NS, records, sec, shadow);
+      if (r != ST_OK) return r;
+      continue;
+    }
+    size_t avail = 0, total = 0;
+    const std::string err = g_err;
+    if (!engine_fits(e, Q, B, NS, records, sec, shadow) &&
+        (cudaMemGetInfo(&avail, &total) != cudaSuccess || s->eng.bytes - e.bytes > (long long)(avail / 4) ||
+         grow_engine(s, e, Q, B, NS, records, sec, shadow) != ST_OK)) {
+      cudaGetLastError();
+      drop_engines(s, k);
+      g_err = err;   // the call goes on
+    }
   }
-  return r;
+  return ST_OK;
 }
 
 void free_edge_records(st_scene* s) {
@@ -801,11 +833,8 @@ int overlap_engines(const st_scene* s, const Plan& p, int Q, bool host_sized, bo
   long long nc = chunk_count(p, Q);
   if (host_sized || timing || nc < 2 || (long long)s->xev.size() < nc + 2 * OVERLAP_ENGINES) return 1;
   int n = 1;
-  while (n < std::min<long long>(nc, s->max_engines) && s->aux_stream[n - 1] && s->eng2[n - 1].Q >= Q &&
-         s->eng2[n - 1].NS >= s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0) &&
-         (p.kind == 0 || (s->eng2[n - 1].records && s->eng2[n - 1].B >= p.B)) &&
-         (!p.sec || s->eng2[n - 1].sec_cap >= (long long)s->eng2[n - 1].B * s->eng2[n - 1].Q) &&
-         (!p.shadow || s->eng2[n - 1].shadow))
+  while (n < std::min<long long>(nc, s->max_engines) && s->aux_stream[n - 1] &&
+         engine_fits(s->eng2[n - 1], Q, p.B, s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0), p.kind == 1, p.sec, p.shadow))
     ++n;
   return n;
 }
@@ -1096,7 +1125,8 @@ st_status plan_call(st_scene* s, const st_view* views, int n_views, int default_
 
 st_status launch_call(st_scene* s, Plan& p, const CallArgs& args, int Q, cudaStream_t st);
 
-st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) {
+// The memory a call needs; engines past the required ones come last.
+st_status reserve(st_scene* s, const Plan& p, int Q, long long chunks) {
   st_status r = ensure_tables(s, (int)p.views.size(), (int)p.segs.size(), p.edges);
   if (r != ST_OK) return r;
   if (p.shadow && (int)p.pairs.size() > s->sh_cap_pairs) {
@@ -1113,10 +1143,47 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
     }
     s->sh_cap_pairs = (int)p.pairs.size();
   }
+  if (p.bins && (r = ensure_bins(s, p)) != ST_OK) return r;
+  if (p.lbins && (r = ensure_light_bins(s)) != ST_OK) return r;
+  if (p.kind == 0 && p.pixels > s->acc_cap) {
+    cudaDeviceSynchronize();
+    drop_graphs(s);
+    dfree(s->acc);
+    dfree(s->sacc);
+    if (dalloc(&s->acc, 6 * (size_t)p.pixels) != cudaSuccess || dalloc(&s->sacc, (size_t)p.pixels) != cudaSuccess) {
+      dfree(s->acc);
+      dfree(s->sacc);
+      cudaGetLastError();
+      s->acc_cap = 0;
+      return fail(ST_ERR_OOM, "forward accumulation buffer");
+    }
+    s->acc_cap = p.pixels;
+  }
+  return ensure_engine(s, Q, p.B, s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0), p.kind == 1, p.sec, p.shadow, chunks);
+}
+
+st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) {
+  long long Q64 = p.o.chunk_paths > 0 ? p.o.chunk_paths : DEFAULT_CHUNK;
+  Q64 = std::min<long long>(Q64, std::max<long long>(p.total, SEG_ALIGN));
+  Q64 = (Q64 + SEG_ALIGN - 1) / SEG_ALIGN * SEG_ALIGN;
+  int Q = (int)Q64;
+  if (p.o.mode == ST_MODE_PER_VIEW) {
+    long long mx = SEG_ALIGN;
+    for (auto& vr : p.view_range) mx = std::max(mx, vr.second - vr.first);
+    Q = (int)std::min<long long>(Q, (mx + SEG_ALIGN - 1) / SEG_ALIGN * SEG_ALIGN);
+  }
+  const bool several = p.o.mode == ST_MODE_BATCHED && !p.o.time_kernels && chunk_count(p, Q) >= 2;
+  const long long chunks = several ? chunk_count(p, Q) : 1;
+  const std::string err = g_err;
+  st_status r = reserve(s, p, Q, chunks);
+  if (r == ST_ERR_OOM && drop_engines(s, OVERLAP_REQUIRED)) {   // what earlier calls could do without goes first
+    g_err = err;
+    r = reserve(s, p, Q, chunks);
+  }
+  if (r != ST_OK) return r;
+  if (p.edges) ensure_edge_records(s, (int)p.views.size());
   std::vector<uint32_t> bkey;
   if (p.bins) {
-    r = ensure_bins(s, p);
-    if (r != ST_OK) return r;
     bkey = bins_key(p);
     // a build whose lists overflowed (as far as its readback shows yet) is redone with more room
     p.bins_reused = s->bins_valid && s->bins_geom == s->geom_version && s->bins_key == bkey &&
@@ -1124,8 +1191,6 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
     if (!p.bins_reused) s->bins_valid = false;
   }
   if (p.lbins) {
-    r = ensure_light_bins(s);
-    if (r != ST_OK) return r;
     p.lbins_reused = s->lbins_valid && s->lbins_geom == s->geom_version &&
                      !(s->lbin_total_host && *s->lbin_total_host > s->lbin_cap);
     if (!p.lbins_reused) s->lbins_valid = false;
@@ -1144,38 +1209,9 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
   }
   p.hz_reused = p.hz && s->hz_valid && s->hz_geom == s->geom_version;
   if (p.hz && !p.hz_reused) s->hz_valid = false;
-  if (p.kind == 0 && p.pixels > s->acc_cap) {
-    cudaDeviceSynchronize();
-    drop_graphs(s);
-    dfree(s->acc);
-    dfree(s->sacc);
-    if (dalloc(&s->acc, 6 * (size_t)p.pixels) != cudaSuccess || dalloc(&s->sacc, (size_t)p.pixels) != cudaSuccess) {
-      dfree(s->acc);
-      dfree(s->sacc);
-      cudaGetLastError();
-      s->acc_cap = 0;
-      return fail(ST_ERR_OOM, "forward accumulation buffer");
-    }
-    s->acc_cap = p.pixels;
-  }
-  long long Q64 = p.o.chunk_paths > 0 ? p.o.chunk_paths : DEFAULT_CHUNK;
-  Q64 = std::min<long long>(Q64, std::max<long long>(p.total, SEG_ALIGN));
-  Q64 = (Q64 + SEG_ALIGN - 1) / SEG_ALIGN * SEG_ALIGN;
-  int Q = (int)Q64;
-  if (p.o.mode == ST_MODE_PER_VIEW) {
-    long long mx = SEG_ALIGN;
-    for (auto& vr : p.view_range) mx = std::max(mx, vr.second - vr.first);
-    Q = (int)std::min<long long>(Q, (mx + SEG_ALIGN - 1) / SEG_ALIGN * SEG_ALIGN);
-  }
-  int NS = s->nl + p.max_vl + (s->env.w > 0 ? 1 : 0);
-  bool timing_call = p.o.time_kernels != 0;
-  bool want_two = p.o.mode == ST_MODE_BATCHED && !timing_call && chunk_count(p, Q) >= 2;
-  r = ensure_engine(s, Q, p.B, NS, p.kind == 1, p.sec, p.shadow, want_two ? chunk_count(p, Q) : 1);
-  if (r != ST_OK) return r;
-  if (p.edges) ensure_edge_records(s, (int)p.views.size());
-  if (want_two) {
+  if (several) {
     // events for the fork, every chunk's resolve and the join, made before any capture
-    long long need = chunk_count(p, Q) + 2 * OVERLAP_ENGINES;
+    long long need = chunks + 2 * OVERLAP_ENGINES;
     while ((long long)s->xev.size() < need) {
       cudaEvent_t e;
       ST_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));

@@ -80,7 +80,7 @@ struct Engine {
 // engines no longer fill the SMs: four took an iteration on 200k faces and 64 views from 35.3 to 32.7 ms, one of 1M
 // faces from 123.5 to 115.0, a two-view preview from 4.58 to 4.12 (six or eight: within 2 % of four).
 constexpr int OVERLAP_ENGINES = 4;
-constexpr int OVERLAP_REQUIRED = 2;   // a call of two chunks or more fails without these; the others are used if they fit
+constexpr int OVERLAP_REQUIRED = 2;   // a call of two chunks or more fails without these; the others are given back where memory is short
 
 enum { CNT_EXT = 0, CNT_EXT_FETCH = 16, CNT_SHADE_FETCH = 32, CNT_SH = 48, CNT_SH_FETCH = 64, CNT_MISC = 80,
        CNT_SEC = CNT_MISC, CNT_FB = 88, CNT_FB_FETCH = 89, CNT_SIZE = 96 };
@@ -209,7 +209,7 @@ struct st_scene {
   st::Engine eng;
   st::Engine eng2[st::OVERLAP_ENGINES - 1];   // further engines: consecutive chunks of a batched call rotate over all
   cudaStream_t aux_stream[st::OVERLAP_ENGINES - 1] = {};   // their streams (join a captured graph through events)
-  int max_engines = st::OVERLAP_ENGINES;   // lowered when a further engine did not fit into memory
+  int max_engines = st::OVERLAP_ENGINES;   // lowered where a further engine did not fit, until the first one grows
   std::vector<cudaEvent_t> xev;  // fork, per-chunk resolve and join events of overlapped calls
   int xev_used = 0;
   int* d_err = nullptr;

@@ -1,4 +1,4 @@
-"""Memory that a call can do without: screen records of edge candidates.
+"""Memory that a call can do without: screen records of edge candidates, wavefront engines past the second.
 
 Where it is short, or would be large, the call runs with less of it and gives the same result.
 """
@@ -84,3 +84,77 @@ def test_edge_records_of_thousands_of_views_stay_small(st):  # noqa: F811
     _close(got, ref)
     scene.close()
     other.close()
+
+
+def _chunked(st, **kw):
+    return st.make_opts(chunk_paths=2048, **kw)   # 9600 paths: five chunks, so four engines where they fit
+
+
+def _image(scene, sc, opts):
+    img = scene.render(sc.views, 2, 7, opts).cpu().numpy()
+    assert scene.stats()["device_error"] == 0
+    return img
+
+
+def test_further_engines_that_do_not_fit_are_done_without(st):  # noqa: F811
+    sc = _small()
+    scene = st.Scene.from_scene(sc)
+    ref = _image(scene, sc, _chunked(st))
+    full = scene.stats()["scratch_bytes"]
+    scene.close()
+    held = []
+    for n in range(120):
+        scene = st.Scene.from_scene(sc)
+        with pytest.raises(st.StError):
+            scene.render([], 2, 7, out=torch.zeros((sc.n_pixels, 3), device="cuda"))
+        said = st.lib().st_last_error()
+        st.inject_fault("alloc", n)
+        try:
+            img = _image(scene, sc, _chunked(st))
+        except st.StError as e:
+            assert e.status == 2
+            st.inject_fault("alloc", -1)
+            np.testing.assert_array_equal(_image(scene, sc, _chunked(st)), ref)
+            scene.close()
+            continue
+        finally:
+            st.inject_fault("alloc", -1)
+        np.testing.assert_array_equal(img, ref)
+        assert st.lib().st_last_error() == said   # nothing was refused
+        held.append(scene.stats()["scratch_bytes"])
+        np.testing.assert_array_equal(_image(scene, sc, _chunked(st)), ref)
+        scene.close()
+        if held[-1] == full:
+            break
+    # first without the third and the fourth engine, then without the fourth, then with all of them
+    assert sorted(set(held)) == [full // 2, full // 4 * 3, full]
+
+
+@pytest.mark.parametrize("backward", [False, True])
+def test_further_engines_are_given_back_where_memory_is_short(st, backward):  # noqa: F811
+    """A later call's buffers do not fit beside the optional engines: they go, and the call succeeds."""
+    sc, big = _small(), S.tiny(res=72, spp=3)
+    big.views = S.ring_views(5, 72, 3)
+    call = _gradient if backward else _image
+    opts = _chunked(st, edge_term=1 if backward else 0)
+    fresh = st.Scene.from_scene(big)
+    ref = call(fresh, big, opts)
+    fresh.close()
+    for n in range(200):
+        scene = st.Scene.from_scene(sc)
+        call(scene, sc, opts)
+        before = scene.stats()["scratch_bytes"]
+        st.inject_fault("alloc", n)
+        try:
+            got = call(scene, big, opts)   # no allocation's failure reaches the caller while engines can be given back
+        finally:
+            st.inject_fault("alloc", -1)
+        (_close if backward else np.testing.assert_array_equal)(got, ref)
+        after = scene.stats()["scratch_bytes"]
+        (_close if backward else np.testing.assert_array_equal)(call(scene, big, opts), ref)
+        scene.close()
+        if n == 0:
+            assert after < before   # the tables came first: two engines stayed
+        st.inject_fault("alloc", -1)
+        if n > 6:
+            return
