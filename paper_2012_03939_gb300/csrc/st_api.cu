@@ -68,25 +68,29 @@ constexpr int EDGE_RECORDS = 1 << 15;
 constexpr long long EDGE_RECORD_BYTES = 256LL << 20;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
-// Whether a call uses the faces' free directions (k_horizon). A face costs 8 (smooth) to 17 ns (rough) to build; of the
-// rays a path can send, those they spare the tree cost about 0.04 ns each (iterations on 5120 faces, B = 3, listed
-// lights only: 0.08 to 0.12 ns a path; 200k faces, B = 3, environment: 0.20; 1M rough ones, B = 5, environment: 0.32).
-// Those are the bounce rays and, where the call has other lights than the listed ones of the scene, the next-event rays;
-// a listed light's rays cost little without. An iteration's two calls share one build, so a call counts from HZ_GAIN
-// such rays per face on. Below HZ_MIN_JOBS paths the two launches' latency (50 us) is not won back; on an open mesh,
-// whose faces mostly see one another (three planes of 384 faces: a third of the cells empty, 0.97x at 786k paths), not
-// below HZ_MIN_JOBS_OPEN.
+// Whether a call uses the faces' free directions (uses_free_directions). A face costs 8 (smooth) to 17 ns (rough) to build; a
+// path wins back what the rays they answer would have cost, which depends on the share of the directions that is free
+// (hz_survey). Paths a face at which iterations with and without them took the same time, environment and bounce rays:
+//   1.00 free (displaced spheres)                22 (one vertex a path: 45)
+//   0.90 to 0.96 (fractal spheres)               50 to 57 (130)
+//   0.41 to 0.46 (torus knots of 12k to 160k)    130 to 250; listed lights alone 300 to 600; traced lights 75 to 125
+//   0.23 to 0.33 (rougher spheres, any size)     none up to 1920 (0.90 to 0.99 of the speed without)
+//   0.28 to 0.33 (three planes, open)            below 480 (1.04 to 1.2 from there on)
+// Rays to the scene's listed lights (see light_bin_range) cost little without, and bounces after the first count for
+// little, since few paths get there: a call of listed lights and one vertex a path loses on any but smooth meshes (0.98 at
+// 480). A build that serves a forward call alone takes twice the paths. Below HZ_MIN_JOBS paths the two launches' latency
+// (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN (three planes of 384 faces: 0.97x at 786k paths).
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
-constexpr int HZ_GAIN = 200;
-// A forward call that no adjoint follows has to win the build back by itself. On gentle surfaces it does from HZ_GAIN on
-// (two-view preview of 200k faces, 250 rays a face: 5.5 -> 4.9 ms); on rough or concave ones a build costs twice as much
-// and spares half: renders alone, with and without the build, of 1M rough faces (300 rays a face) 39.2 and 27.2 ms, of
-// 249k (315) 12.2 and 11.0, of a 50k-face torus knot (1170) 4.60 and 4.39; of one of 36k faces (4200) 7.65 with, 8.75
-// before there were any. So HZ_GAIN_ROUGH is asked of these. The surface is gentle while the sines by which neighbours
-// rise above a face average below HZ_GENTLE (displaced spheres 0 to 2e-5, torus knot 0.0097, rough 0.022), as the scene
-// was created; an adjoint follows if one did on these vertices or the last.
-constexpr int HZ_GAIN_ROUGH = 1600;
-constexpr double HZ_GENTLE = 0.002;
+constexpr double HZ_SMOOTH = 0.95, HZ_FRACTAL = 0.7, HZ_CONCAVE = 0.35;   // least shares of free directions
+constexpr int HZ_PATHS_SMOOTH = 22, HZ_PATHS_FRACTAL = 60, HZ_PATHS_CONCAVE = 140, HZ_PATHS_CONCAVE_LISTED = 400,
+              HZ_PATHS_CONCAVE_TRACED = 110, HZ_PATHS_OPEN = 400;
+constexpr double HZ_ALONE = 2.0;
+// Longest edge from which no direction is usable: the directions' margins grow with it (by a tenth of its length in the sine
+// of elevation, T_EPS being fixed). What a smooth sphere of 20k faces and 256 rays a face won, 0.48 ms of the 1.26 an
+// iteration takes at a longest edge of 0.05, was 0.33 at 1, 0.14 at 3, 0.06 at 5 and nothing at 8.5 (the build takes
+// 0.17): the square of 1 - edge / HZ_LONGEST.
+constexpr double HZ_LONGEST = 8.0;
+constexpr int HZ_SURVEY = 1024;   // faces that the share of free directions is taken from
 // Segment bases and chunk sizes are multiples of 64: an edge segment is laid out
 // in blocks of 64 jobs, the minus sides of 32 consecutive samples then their plus
 // sides, so every warp traces one side along one edge (same behaviour per lane).
@@ -210,40 +214,6 @@ void build_edges(const std::vector<int>& F, int nf, std::vector<int2>& ev, std::
     ef.push_back(make_int2(e[i].second, second));
     i = j;
   }
-}
-
-// Mean over the edges of two faces of the sine by which the second face rises above the plane of the first, on the
-// outer side of a closed mesh (0 where it falls away).
-double mean_rise(const std::vector<float>& V, const std::vector<int>& F, int nf, const std::vector<int2>& ev,
-                 const std::vector<int2>& ef) {
-  auto at = [&](int v, double (&x)[3]) { for (int k = 0; k < 3; ++k) x[k] = V[3 * (size_t)v + k]; };
-  auto normal = [&](int f, double (&n)[3], double (&a)[3]) {
-    double b[3], c[3];
-    at(F[3 * f], a); at(F[3 * f + 1], b); at(F[3 * f + 2], c);
-    for (int k = 0; k < 3; ++k) { b[k] -= a[k]; c[k] -= a[k]; }
-    for (int k = 0; k < 3; ++k) n[k] = b[(k + 1) % 3] * c[(k + 2) % 3] - b[(k + 2) % 3] * c[(k + 1) % 3];
-  };
-  auto len = [](const double (&x)[3]) { return std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]); };
-  double vol = 0.0, n[3], a[3];
-  for (int f = 0; f < nf; ++f) {
-    normal(f, n, a);
-    vol += n[0] * a[0] + n[1] * a[1] + n[2] * a[2];
-  }
-  double sum = 0.0;
-  size_t cnt = 0;
-  for (size_t i = 0; i < ef.size(); ++i) {
-    if (ef[i].y < 0) continue;
-    const int* g = &F[3 * (size_t)ef[i].y];
-    const int apex = g[0] != ev[i].x && g[0] != ev[i].y ? g[0] : g[1] != ev[i].x && g[1] != ev[i].y ? g[1] : g[2];
-    double x[3], b[3];
-    normal(ef[i].x, n, a);
-    at(apex, x); at(ev[i].x, b);
-    for (int k = 0; k < 3; ++k) x[k] -= b[k];
-    const double h = (vol < 0.0 ? -1.0 : 1.0) * (n[0] * x[0] + n[1] * x[1] + n[2] * x[2]), l = len(n) * len(x);
-    if (h > 0.0 && l > 0.0) sum += h / l;
-    ++cnt;
-  }
-  return cnt ? sum / (double)cnt : 0.0;
 }
 
 // True when the faces form one connected surface (across shared edges) in
@@ -595,17 +565,45 @@ std::vector<uint32_t> bins_key(const Plan& p) {
   return k;
 }
 
-// the faces' free directions on the current vertices
-cudaError_t hz_build(st_scene* s, cudaStream_t st) {
+// the free directions of every stride-th face on the current vertices
+cudaError_t hz_build(st_scene* s, cudaStream_t st, int stride = 1) {
   if (s->n4 > 0) {
     cudaError_t e = cudaMemsetAsync(s->hz_done, 0, sizeof(int) * s->n4, st);
     if (e != cudaSuccess) return e;
     k_hz_nodes<<<(s->n4 + 127) / 128, 128, 0, st>>>(s->nodes4, s->tri, s->parent4, s->n4, s->nf, s->mstat, s->hz_nodes,
                                                     s->hz_done, s->d_err);
   }
-  k_horizon<<<(s->nf + HZ_WARPS - 1) / HZ_WARPS, 32 * HZ_WARPS, 0, st>>>(
-      s->nodes4, s->tri, s->nf, s->n4, s->mstat, s->hz_nodes, s->parent4, s->leaf_node4, s->hz, s->d_err);
+  const int n = (s->nf + stride - 1) / stride;
+  k_horizon<<<(n + HZ_WARPS - 1) / HZ_WARPS, 32 * HZ_WARPS, 0, st>>>(
+      s->nodes4, s->tri, s->nf, s->n4, s->mstat, s->hz_nodes, s->parent4, s->leaf_node4, s->hz, s->d_err, stride);
   return cudaGetLastError();
+}
+
+// What the free directions would answer, from some of the faces: the share of cosine-distributed directions, and how far the
+// longest edge leaves it usable. Taken once, by the scene's first call that is large enough for them (0.15 ms, most of it one
+// warp's walk); waits for the stream. The cells are not those of a build.
+cudaError_t hz_survey(st_scene* s, cudaStream_t st) {
+  s->hz_valid = false;
+  const int stride = std::max(1, s->nf / HZ_SURVEY);
+  cudaError_t e = hz_build(s, st, stride);
+  std::vector<uint4> cells((s->nf + stride - 1) / stride);
+  MeshStat ms;
+  if (e == cudaSuccess) e = copy_async(cells.data(), s->hz, sizeof(uint4) * cells.size(), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = copy_async(&ms, s->mstat, sizeof(ms), cudaMemcpyDeviceToHost, st);
+  const cudaError_t w = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = w;
+  if (e != cudaSuccess) return e;
+  double share[16], free = 0.0;
+  for (int b = 0; b < 16; ++b) {
+    const double lo = b == 0 ? HZ_FLOOR : HZ_LOW + (b - 1) * (1.0 - HZ_LOW) / 15.0, hi = HZ_LOW + b * (1.0 - HZ_LOW) / 15.0;
+    share[b] = (hi * hi - lo * lo) / 8.0;
+  }
+  for (const uint4& c : cells)
+    for (unsigned w : {c.x, c.y, c.z, c.w})
+      for (int k = 0; k < 32; ++k) free += w >> k & 1u ? 0.0 : share[k & 15];
+  s->hz_free = free / (double)cells.size();
+  s->hz_reach = std::max(0.0, 1.0 - ms.eta * 1e6 / HZ_LONGEST);
+  return cudaSuccess;
 }
 
 KCtx make_ctx(st_scene* s, const Plan& p) {
@@ -1125,6 +1123,26 @@ st_status plan_call(st_scene* s, const st_view* views, int n_views, int default_
 
 st_status launch_call(st_scene* s, Plan& p, const CallArgs& args, int Q, cudaStream_t st);
 
+// The rule of HZ_MIN_JOBS and the constants beside it. An adjoint and the forward call before it share one build: a forward
+// call expects its adjoint if one ran on these vertices or the last.
+bool uses_free_directions(const st_scene* s, const Plan& p) {
+  if (p.total < (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN)) return false;
+  const bool env = s->env.w > 0, traced = p.max_vl > 0 || (s->nl > 0 && !p.lbins), smooth = s->hz_free >= HZ_SMOOTH,
+             fractal = s->hz_free >= HZ_FRACTAL, built = s->hz_valid && s->hz_geom == s->geom_version;
+  if (built && fractal) return true;   // as the call that built them decided
+  if (s->closed && s->hz_free < HZ_CONCAVE) return false;
+  if (p.B == 1 && !env && !traced && !smooth) return false;
+  double need = smooth ? HZ_PATHS_SMOOTH : fractal ? HZ_PATHS_FRACTAL : !s->closed ? HZ_PATHS_OPEN : traced ? HZ_PATHS_CONCAVE_TRACED
+              : env ? HZ_PATHS_CONCAVE : HZ_PATHS_CONCAVE_LISTED;
+  if (p.B == 1 && !traced) need *= env ? 2.0 : 8.0;
+  double paths = (double)p.total;
+  if (p.kind == 0 && !built) {
+    if (s->adj_seen && s->geom_version - s->adj_geom <= 1) paths = 0.5 * (paths + (double)s->adj_total);
+    else need *= HZ_ALONE;
+  }
+  return paths * s->hz_reach * s->hz_reach >= need * s->nf;
+}
+
 // The memory a call needs; engines past the required ones come last.
 st_status reserve(st_scene* s, const Plan& p, int Q, long long chunks) {
   st_status r = ensure_tables(s, (int)p.views.size(), (int)p.segs.size(), p.edges);
@@ -1195,17 +1213,15 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
                      !(s->lbin_total_host && *s->lbin_total_host > s->lbin_cap);
     if (!p.lbins_reused) s->lbins_valid = false;
   }
-  {
-    const bool unlisted = s->env.w > 0 || p.max_vl > 0 || (s->nl > 0 && !p.lbins);
-    const double rays = (p.B - 1) + (unlisted ? p.B : 0.25);   // per path
-    const bool built = s->hz_valid && s->hz_geom == s->geom_version;
-    const bool alone = p.kind == 0 && !built && !s->gentle && !(s->adj_seen && s->geom_version - s->adj_geom <= 1);
-    p.hz = p.total >= (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN) &&
-           rays * (double)p.total >= (double)(alone ? HZ_GAIN_ROUGH : HZ_GAIN) * s->nf;
-    if (p.kind == 1) {
-      s->adj_seen = true;
-      s->adj_geom = s->geom_version;
-    }
+  if (s->hz_free < 0.0 && p.total >= HZ_MIN_JOBS) {
+    const cudaError_t e = hz_survey(s, st);
+    if (e != cudaSuccess) return cuda_fail(e, "survey of the free directions");
+  }
+  p.hz = uses_free_directions(s, p);
+  if (p.kind == 1) {
+    s->adj_seen = true;
+    s->adj_geom = s->geom_version;
+    s->adj_total = p.total;
   }
   p.hz_reused = p.hz && s->hz_valid && s->hz_geom == s->geom_version;
   if (p.hz && !p.hz_reused) s->hz_valid = false;
@@ -1402,7 +1418,6 @@ st_status st_scene_create(const st_scene_desc* d, void* stream, st_scene** out) 
   std::vector<int2> ev, ef;
   build_edges(hf, s->nf, ev, ef);
   s->closed = closed_single_surface(hf, s->nf, ef);
-  s->gentle = mean_rise(hv, hf, s->nf, ev, ef) < HZ_GENTLE;
   s->n_edges = (int)ev.size();
   std::vector<float4> etex;
   std::vector<float2> etab;

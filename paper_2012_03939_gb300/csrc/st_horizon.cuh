@@ -408,15 +408,17 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
                                                            const float4* __restrict__ tri, int nf, int n4,
                                                            const MeshStat* ms, const float4* __restrict__ N,
                                                            const int* parent, const int* leaf_node, uint4* out,
-                                                           int* err) {
+                                                           int* err, int stride) {
   __shared__ int stack_[HZ_WARPS][HZ_STACK], cand_[HZ_WARPS][64];
   __shared__ float lines_[HZ_WARPS][18];   // f's border lines (mx, my, mo): the finer bound's alone, kept off the registers
   const unsigned ALL = 0xffffffffu;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   int *stack = stack_[warp], *cand = cand_[warp];
-  const int li = blockIdx.x * HZ_WARPS + warp;
-  if (li >= nf) return;
+  const int place = blockIdx.x * HZ_WARPS + warp;
+  const long long leaf = (long long)place * stride;   // every stride-th face, its cells one after the other
+  if (leaf >= nf) return;
+  const int li = (int)leaf;
   const float side = ms->winding < 0 ? -1.0f : 1.0f;
   HzFace f;
   const bool bad = !hz_face(xyz(tri[3 * li]), xyz(tri[3 * li + 1]), xyz(tri[3 * li + 2]), side, f);
@@ -512,7 +514,7 @@ __global__ void __launch_bounds__(32 * HZ_WARPS, 3) k_horizon(const float4* __re
       if (last) break;
     }
   }
-  if (lane == 0) out[li] = bad ? make_uint4(ALL, ALL, ALL, ALL) : make_uint4(M[0], M[1], M[2], M[3]);
+  if (lane == 0) out[place] = bad ? make_uint4(ALL, ALL, ALL, ALL) : make_uint4(M[0], M[1], M[2], M[3]);
 }
 
 // The free directions of a path vertex p on the face (v0, v1, v2) with the marked cells w; n: its unit normal turned

@@ -195,9 +195,10 @@ struct st_scene {
   cudaEvent_t hz_ev[2] = {};               // its fork and join
   bool hz_valid = false;
   unsigned long long hz_geom = 0;
-  bool gentle = false;           // neighbouring faces hardly rise above one another (mean_rise)
-  bool adj_seen = false;         // geom_version of the last adjoint call
-  unsigned long long adj_geom = 0;
+  double hz_free = -1, hz_reach = 0;       // hz_survey's (-1: not taken yet)
+  bool adj_seen = false;         // an adjoint call was made,
+  unsigned long long adj_geom = 0;         // the last one on this geom_version,
+  long long adj_total = 0;                 // of so many paths
   float* acc = nullptr;          // [6 * pixels] forward accumulation, compensated FP32 (sum, error) per channel
   unsigned long long* sacc = nullptr;  // [pixels] path-signature sums (bin-space pixel index)
   long long acc_cap = 0;

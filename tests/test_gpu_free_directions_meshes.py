@@ -66,15 +66,15 @@ def test_moved_and_scaled_meshes(st, mesh, where, scale):  # noqa: F811
         V = S.sinusoid_displace(V, rng, amp=0.3)
     elif mesh == "rough":
         V, F = S.uv_sphere(60, 31)
-        V = S.fractal_displace(V, rng, amp=0.4)
+        V = S.fractal_displace(V, rng, amp=0.12)
     else:
-        V, F = S.torus_knot(2, 3, 120, 16)
+        V, F = S.torus_knot(2, 3, 120, 12)   # 2880 faces: 190 paths each, a concave mesh uses them from 140 on
     at = where * np.array([1.0, -0.7, 0.4])
     sc = _scene(V * scale + at, F, _views(True, at, scale), rng)
     scene = st.Scene.from_scene(sc)
     many, few = _equal_to_small_calls(st, scene, sc)
-    if mesh == "sphere" and (where, scale) in ((10.0, 1.0), (0.0, 1e-3)):
-        assert many["node_visits"] + many["shadow_node_visits"] < 0.9 * (few["node_visits"] + few["shadow_node_visits"])
+    if (where, scale) in ((10.0, 1.0), (100.0, 0.05)):   # longest edges below a unit, vertices near enough to their faces
+        assert many["node_visits"] + many["shadow_node_visits"] < 0.97 * (few["node_visits"] + few["shadow_node_visits"])
     scene.close()
 
 

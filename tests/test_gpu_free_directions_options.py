@@ -27,7 +27,7 @@ def _scene(opt, light, seed):
     brdf, fresnel, rgb, res, smooth = opt
     rng = np.random.default_rng(seed)
     V, F = S.uv_sphere(60, 31)
-    V = S.fractal_displace(V, rng, amp=0.4)
+    V = S.fractal_displace(V, rng, amp=0.12)
     P = S.random_face_params(rng, len(F) * (res + 1) * (res + 2) // 2)
     if rgb:
         P = np.concatenate([P[:, :3], rng.uniform(0.02, 0.3, size=(len(P), 3)).astype(np.float32), P[:, 4:]], 1)
