@@ -69,22 +69,24 @@ constexpr long long EDGE_RECORD_BYTES = 256LL << 20;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
 // Whether a call uses the faces' free directions (uses_free_directions). A face costs 8 (smooth) to 17 ns (rough) to build; a
-// path wins back what the rays they answer would have cost, which depends on the share of the directions that is free
-// (hz_survey). Paths a face at which iterations with and without them took the same time, environment and bounce rays:
-//   1.00 free (displaced spheres)                22 (one vertex a path: 45)
-//   0.90 to 0.96 (fractal spheres)               50 to 57 (130)
-//   0.41 to 0.46 (torus knots of 12k to 160k)    130 to 250; listed lights alone 300 to 600; traced lights 75 to 125
-//   0.23 to 0.33 (rougher spheres, any size)     none up to 1920 (0.90 to 0.99 of the speed without)
-//   0.28 to 0.33 (three planes, open)            below 480 (1.04 to 1.2 from there on)
+// path that hits the mesh wins back what the rays they answer would have cost, which depends on the share of the directions
+// that is free (hz_survey). Hits a face (expected_hits) at which iterations with and without them took the same time,
+// environment and bounce rays:
+//   1.00 free (displaced spheres)                12 (one vertex a path: 26)
+//   0.90 to 0.96 (fractal spheres)               30 to 34 (75)
+//   0.41 to 0.46 (torus knots of 12k to 160k)    50 to 100; listed lights alone 120 to 240; traced lights 30 to 50
+//   0.23 to 0.33 (rougher spheres, any size)     none up to 1500 (0.90 to 0.99 of the speed without)
+//   0.28 to 0.33 (three planes, open)            below 270 (1.04 to 1.2 from there on)
 // Rays to the scene's listed lights (see light_bin_range) cost little without, and bounces after the first count for
 // little, since few paths get there: a call of listed lights and one vertex a path loses on any but smooth meshes (0.98 at
-// 480). A build that serves a forward call alone takes twice the paths. Below HZ_MIN_JOBS paths the two launches' latency
-// (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN (three planes of 384 faces: 0.97x at 786k paths).
+// 280). A build that serves a forward call alone takes half as much again, on concave meshes twice. Below HZ_MIN_JOBS paths
+// the two launches' latency (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN (three planes of 384
+// faces: 0.97x at 786k paths).
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
 constexpr double HZ_SMOOTH = 0.95, HZ_FRACTAL = 0.7, HZ_CONCAVE = 0.35;   // least shares of free directions
-constexpr int HZ_PATHS_SMOOTH = 22, HZ_PATHS_FRACTAL = 60, HZ_PATHS_CONCAVE = 140, HZ_PATHS_CONCAVE_LISTED = 400,
-              HZ_PATHS_CONCAVE_TRACED = 110, HZ_PATHS_OPEN = 400;
-constexpr double HZ_ALONE = 2.0;
+constexpr int HZ_HITS_SMOOTH = 13, HZ_HITS_FRACTAL = 35, HZ_HITS_CONCAVE = 52, HZ_HITS_CONCAVE_LISTED = 160,
+              HZ_HITS_CONCAVE_TRACED = 44, HZ_HITS_OPEN = 230;
+constexpr double HZ_ALONE = 1.5, HZ_ALONE_CONCAVE = 2.0;
 // Longest edge from which no direction is usable: the directions' margins grow with it (by a tenth of its length in the sine
 // of elevation, T_EPS being fixed). What a smooth sphere of 20k faces and 256 rays a face won, 0.48 ms of the 1.26 an
 // iteration takes at a longest edge of 0.05, was 0.33 at 1, 0.14 at 3, 0.06 at 5 and nothing at 8.5 (the build takes
@@ -601,6 +603,13 @@ cudaError_t hz_survey(st_scene* s, cudaStream_t st) {
   for (const uint4& c : cells)
     for (unsigned w : {c.x, c.y, c.z, c.w})
       for (int k = 0; k < 32; ++k) free += w >> k & 1u ? 0.0 : share[k & 15];
+  double d2 = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    const double lo = from_ordered(ms.lo[k]), hi = from_ordered(ms.hi[k]);
+    s->hz_mid[k] = 0.5 * (lo + hi);
+    d2 += (hi - lo) * (hi - lo) / 3.0;
+  }
+  s->hz_radius = 0.5 * std::sqrt(d2);
   s->hz_free = free / (double)cells.size();
   s->hz_reach = std::max(0.0, 1.0 - ms.eta * 1e6 / HZ_LONGEST);
   return cudaSuccess;
@@ -1123,24 +1132,47 @@ st_status plan_call(st_scene* s, const st_view* views, int n_views, int default_
 
 st_status launch_call(st_scene* s, Plan& p, const CallArgs& args, int Q, cudaStream_t st);
 
+// About how many of a call's paths hit the mesh: of a view's camera samples those within the disk that a sphere of the
+// mesh's mean extent covers (views of 407 x 54 pixels show it in a fifteenth), and of the edges' sides every other one.
+double expected_hits(const st_scene* s, const Plan& p, bool camera_only) {
+  double hits = 0.0;
+  for (const Seg& sg : p.segs) {
+    if (sg.kind != 0) { hits += camera_only ? 0.0 : 0.5 * (double)sg.count; continue; }
+    const DevView& v = p.views[sg.view];
+    const double e[3] = {s->hz_mid[0] - v.eye.x, s->hz_mid[1] - v.eye.y, s->hz_mid[2] - v.eye.z};
+    const double d2 = e[0] * e[0] + e[1] * e[1] + e[2] * e[2] - s->hz_radius * s->hz_radius;
+    double part = 1.0;
+    if (d2 > 0.0) {
+      const double t = s->hz_radius / std::sqrt(d2);   // tangent of the half angle it is seen under
+      part = std::min(1.0, t / v.kx) * std::min(1.0, t / v.ky) * 0.7854;
+    }
+    hits += part * (double)sg.count;
+  }
+  return hits;
+}
+
 // The rule of HZ_MIN_JOBS and the constants beside it. An adjoint and the forward call before it share one build: a forward
 // call expects its adjoint if one ran on these vertices or the last.
 bool uses_free_directions(const st_scene* s, const Plan& p) {
-  if (p.total < (s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN)) return false;
+  const long long least = s->closed ? HZ_MIN_JOBS : HZ_MIN_JOBS_OPEN;
+  if (p.total < least) return false;
   const bool env = s->env.w > 0, traced = p.max_vl > 0 || (s->nl > 0 && !p.lbins), smooth = s->hz_free >= HZ_SMOOTH,
              fractal = s->hz_free >= HZ_FRACTAL, built = s->hz_valid && s->hz_geom == s->geom_version;
   if (built && fractal) return true;   // as the call that built them decided
   if (s->closed && s->hz_free < HZ_CONCAVE) return false;
   if (p.B == 1 && !env && !traced && !smooth) return false;
-  double need = smooth ? HZ_PATHS_SMOOTH : fractal ? HZ_PATHS_FRACTAL : !s->closed ? HZ_PATHS_OPEN : traced ? HZ_PATHS_CONCAVE_TRACED
-              : env ? HZ_PATHS_CONCAVE : HZ_PATHS_CONCAVE_LISTED;
+  double need = smooth ? HZ_HITS_SMOOTH : fractal ? HZ_HITS_FRACTAL : !s->closed ? HZ_HITS_OPEN : traced ? HZ_HITS_CONCAVE_TRACED
+              : env ? HZ_HITS_CONCAVE : HZ_HITS_CONCAVE_LISTED;
   if (p.B == 1 && !traced) need *= env ? 2.0 : 8.0;
-  double paths = (double)p.total;
-  if (p.kind == 0 && !built) {
-    if (s->adj_seen && s->geom_version - s->adj_geom <= 1) paths = 0.5 * (paths + (double)s->adj_total);
-    else need *= HZ_ALONE;
+  double hits = expected_hits(s, p, false);
+  if (!built) {   // the mean of the two calls, none for one too small to use them; a call alone asks HZ_ALONE times as much
+    long long camera = 0;
+    for (const Seg& sg : p.segs) camera += sg.kind == 0 ? sg.count : 0;
+    if (p.kind == 1) hits = 0.5 * (hits + (camera >= least ? expected_hits(s, p, true) : 0.0));
+    else if (s->adj_seen && s->geom_version - s->adj_geom <= 1) hits = 0.5 * (hits + s->adj_hits);
+    else need *= fractal ? HZ_ALONE : HZ_ALONE_CONCAVE;
   }
-  return paths * s->hz_reach * s->hz_reach >= need * s->nf;
+  return hits * s->hz_reach * s->hz_reach >= need * s->nf;
 }
 
 // The memory a call needs; engines past the required ones come last.
@@ -1221,7 +1253,7 @@ st_status run_call(st_scene* s, Plan& p, const CallArgs& args, cudaStream_t st) 
   if (p.kind == 1) {
     s->adj_seen = true;
     s->adj_geom = s->geom_version;
-    s->adj_total = p.total;
+    s->adj_hits = expected_hits(s, p, false);
   }
   p.hz_reused = p.hz && s->hz_valid && s->hz_geom == s->geom_version;
   if (p.hz && !p.hz_reused) s->hz_valid = false;

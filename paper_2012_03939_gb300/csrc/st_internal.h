@@ -195,10 +195,11 @@ struct st_scene {
   cudaEvent_t hz_ev[2] = {};               // its fork and join
   bool hz_valid = false;
   unsigned long long hz_geom = 0;
-  double hz_free = -1, hz_reach = 0;       // hz_survey's (-1: not taken yet)
+  double hz_free = -1, hz_reach = 0;       // hz_survey's (-1: not taken yet), with the middle and mean radius of the bounds
+  double hz_mid[3] = {}, hz_radius = 0;
   bool adj_seen = false;         // an adjoint call was made,
   unsigned long long adj_geom = 0;         // the last one on this geom_version,
-  long long adj_total = 0;                 // of so many paths
+  double adj_hits = 0;                     // of so many hits
   float* acc = nullptr;          // [6 * pixels] forward accumulation, compensated FP32 (sum, error) per channel
   unsigned long long* sacc = nullptr;  // [pixels] path-signature sums (bin-space pixel index)
   long long acc_cap = 0;

@@ -508,7 +508,12 @@ __device__ __forceinline__ bool pixel_may_overlap(const ScreenTri& et, int x, in
   return true;
 }
 
-__device__ __forceinline__ float from_ordered(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
+__host__ __device__ __forceinline__ float from_ordered(int i) {
+  i = i >= 0 ? i : i ^ 0x7fffffff;
+  float f;
+  memcpy(&f, &i, sizeof(f));
+  return f;
+}
 
 // A closed, consistently wound surface seen from an eye outside its bounds is
 // first hit on a face wound toward the eye (outward when the signed volume is

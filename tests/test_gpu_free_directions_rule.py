@@ -18,25 +18,26 @@ PATHS = 4 * 128 * 128 * 9   # 589824: above 2^19
 
 def _mesh(name):
     rng = np.random.default_rng(1)
+    # the spheres cover 0.58 of a square view, the knots about 0.4
     if name == "smooth":            # every direction free but the lowest
-        V, F = S.icosphere(5)       # 20480 faces: 28.8 paths each
+        V, F = S.icosphere(5)       # 20480 faces: 16.7 hits each
         return S.sinusoid_displace(V, rng), F
-    if name == "fine fractal":      # 25600 faces: 23 paths each
+    if name == "fine fractal":      # 25600 faces: 14 hits each
         V, F = S.uv_sphere(160, 81)
         return S.fractal_displace(V, np.random.default_rng(7)), F
-    if name == "knot":              # 0.41 free; 3840 faces: 154 paths each
+    if name == "knot":              # 0.41 free; 3840 faces: 60 hits each
         return S.torus_knot(2, 3, 120, 16)
-    if name == "small knot":        # 1536 faces: 384 paths each
+    if name == "small knot":        # 1536 faces: 150 hits each
         return S.torus_knot(2, 3, 128, 6)
-    assert name == "rough"          # 0.3 free; 1600 faces: 369 paths each
+    assert name == "rough"          # 0.3 free; 1600 faces: 290 hits each
     V, F = S.uv_sphere(40, 21)
     return S.fractal_displace(V, np.random.default_rng(7), amp=0.4), F
 
 
-def _builds(st, mesh, light, B, scale, adjoint):
+def _builds(st, mesh, light, B, scale, adjoint, w=128, h=128):
     V, F = _mesh(mesh)
     rng = np.random.default_rng(2)
-    views = S.fibonacci_views(4, [128] * 4, [128] * 4, [9] * 4)
+    views = S.fibonacci_views(4, [w] * 4, [h] * 4, [9] * 4)
     if light == "view":
         views = S.with_view_lights(views)
     for v in views:
@@ -63,7 +64,7 @@ def _builds(st, mesh, light, B, scale, adjoint):
 
 @pytest.mark.parametrize("mesh,light,B,scale,adjoint,builds", [
     ("smooth", "env", 3, 1.0, True, True), ("smooth", "env", 1, 1.0, True, False), ("smooth", "view", 1, 1.0, True, True),
-    ("smooth", "env", 3, 1.0, False, False),      # alone: 28.8 paths a face are not 44
+    ("smooth", "env", 3, 1.0, False, False),      # alone: 16.7 hits a face are not 19.5
     ("smooth", "env", 3, 30.0, True, False),      # edges over a unit long: the margins take too much
     ("fine fractal", "env", 3, 1.0, True, False), ("fine fractal", "view", 3, 1.0, True, False),
     ("knot", "env", 3, 1.0, True, True), ("knot", "env", 1, 1.0, True, False), ("knot", "env", 3, 1.0, False, False),
@@ -95,3 +96,9 @@ def test_a_forward_call_counts_on_its_adjoint(st):  # noqa: F811
     scene.refit(W)
     assert launches() == used + 2 and used == plain
     scene.close()
+
+
+def test_paths_that_miss_do_not_count(st):  # noqa: F811
+    """As many paths in wide views, most of which look past the mesh."""
+    assert _builds(st, "smooth", "env", 3, 1.0, True)
+    assert not _builds(st, "smooth", "env", 3, 1.0, True, w=512, h=32)

@@ -20,11 +20,14 @@ B, SEED = 3, 23
 def _vertices(base, seed):
     """The base mesh with noise of the seed: rough, so that some rays are free and some hit."""
     rng = np.random.default_rng(seed)
-    return S._f32(base * (1.0 + 0.04 * rng.normal(size=(len(base), 1))) + 0.3 * rng.normal(size=3))
+    return S._f32(base * (1.0 + 0.004 * rng.normal(size=(len(base), 1))) + 0.3 * rng.normal(size=3))
 
 
 def _step(scene, sc, w):
     dV, dF = scene.backward(sc.views, B, SEED, w, _opts())
+    built = scene.stats()["kernel_launches"]
+    scene.backward(sc.views, B, SEED, w, _opts())
+    assert built - scene.stats()["kernel_launches"] == 6 + 2   # primary lists and free directions were built, and then kept
     sig = torch.zeros(sc.n_pixels, dtype=torch.int64, device="cuda")
     img = scene.render(sc.views, B, SEED, signatures=sig)
     s = scene.stats()
