@@ -569,8 +569,12 @@ std::vector<uint32_t> bins_key(const Plan& p) {
 
 // the free directions of every stride-th face on the current vertices
 cudaError_t hz_build(st_scene* s, cudaStream_t st, int stride = 1) {
+  cudaError_t e = cudaMemsetAsync(&s->mstat->eta, 0, sizeof(float), st);
+  if (e != cudaSuccess) return e;
+  k_longest_edge<<<std::min((s->nf + HZ_EDGE_BLOCK - 1) / HZ_EDGE_BLOCK, 4 * std::max(s->sm_count, 1)), HZ_EDGE_BLOCK, 0, st>>>(
+      s->tri, s->nf, s->mstat);
   if (s->n4 > 0) {
-    cudaError_t e = cudaMemsetAsync(s->hz_done, 0, sizeof(int) * s->n4, st);
+    e = cudaMemsetAsync(s->hz_done, 0, sizeof(int) * s->n4, st);
     if (e != cudaSuccess) return e;
     k_hz_nodes<<<(s->n4 + 127) / 128, 128, 0, st>>>(s->nodes4, s->tri, s->parent4, s->n4, s->nf, s->mstat, s->hz_nodes,
                                                     s->hz_done, s->d_err);
@@ -946,7 +950,7 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
       ST_CUDA(cudaStreamWaitEvent(st, s->hz_ev[1], 0));
     }
     ST_CUDA(e);
-    s->launches += s->n4 > 0 ? 2 : 1;
+    s->launches += s->n4 > 0 ? 3 : 2;
   }
   // Batched calls of several chunks rotate them over the engines, each on its own
   // stream, so one chunk's last, sparsely filled bounces and launch tails overlap

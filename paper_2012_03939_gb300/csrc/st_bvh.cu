@@ -685,7 +685,6 @@ int sort_blocks_for(int n) { return (n + RS_TILE - 1) / RS_TILE; }
 __global__ void k_mesh_stat_init(MeshStat* m) {
   m->vol6 = 0.0;
   m->winding = 0;
-  m->lmax2 = 0;
   for (int k = 0; k < 3; ++k) {
     m->lo[k] = 0x7fffffff;
     m->hi[k] = (int)0x80000000;
@@ -695,26 +694,16 @@ __global__ void k_mesh_stat_init(MeshStat* m) {
 __global__ void k_mesh_stat(const float* V, int nv, const int* F, int nf, MeshStat* m) {
   __shared__ double sv[8];
   double v = 0.0;
-  float l2 = 0.0f;
   for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
     const int* fi = F + 3 * f;
-    float3 p0 = mk3(V[3 * fi[0]], V[3 * fi[0] + 1], V[3 * fi[0] + 2]), p1 = mk3(V[3 * fi[1]], V[3 * fi[1] + 1], V[3 * fi[1] + 2]),
-           p2 = mk3(V[3 * fi[2]], V[3 * fi[2] + 1], V[3 * fi[2] + 2]);
-    l2 = fmaxf(l2, fmaxf(dot3(p1 - p0, p1 - p0), fmaxf(dot3(p2 - p0, p2 - p0), dot3(p2 - p1, p2 - p1))));
     double a[3], b[3], c[3];
     for (int k = 0; k < 3; ++k) {
       a[k] = V[3 * fi[0] + k]; b[k] = V[3 * fi[1] + k]; c[k] = V[3 * fi[2] + k];
     }
     v += a[0] * (b[1] * c[2] - b[2] * c[1]) - a[1] * (b[0] * c[2] - b[2] * c[0]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    v += __shfl_xor_sync(0xffffffffu, v, o);
-    l2 = fmaxf(l2, __shfl_xor_sync(0xffffffffu, l2, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sv[threadIdx.x >> 5] = v;
-    atomicMax(&m->lmax2, __float_as_int(l2));
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
@@ -745,7 +734,6 @@ __global__ void k_mesh_stat_final(MeshStat* m) {
   double d[3];
   for (int k = 0; k < 3; ++k) d[k] = (double)unordered(m->hi[k]) - (double)unordered(m->lo[k]);
   double box6 = 6.0 * d[0] * d[1] * d[2];
-  m->eta = 1e-6f * sqrtf(__int_as_float(m->lmax2));
   m->winding = fabs(m->vol6) > 1e-3 * box6 ? (m->vol6 > 0.0 ? 1 : -1) : 0;
 }
 

@@ -160,6 +160,24 @@ __device__ __forceinline__ float hz_support(const HzNode& q, float3 n) {
   return fminf(q.R, (ct >= 0.0f ? ct * q.smax : ct * q.smin) + st * q.R);
 }
 
+// Raises ms->eta (zeroed before) to 1e-6 of the mesh's longest edge, for what uses the cells. Part of the build, since only
+// that needs it: in the mesh facts of every vertex update an atomic a warp cost 4 us of a 65k-face refit.
+constexpr int HZ_EDGE_BLOCK = 256;
+__global__ void __launch_bounds__(HZ_EDGE_BLOCK) k_longest_edge(const float4* __restrict__ tri, int nf, MeshStat* ms) {
+  __shared__ float part[HZ_EDGE_BLOCK / 32];
+  float l2 = 0.0f;
+  for (int i = blockIdx.x * HZ_EDGE_BLOCK + threadIdx.x; i < nf; i += gridDim.x * HZ_EDGE_BLOCK) {
+    const float3 a = xyz(tri[3 * i]), b = xyz(tri[3 * i + 1]) - a, c = xyz(tri[3 * i + 2]) - a, d = c - b;
+    l2 = fmaxf(l2, fmaxf(dot3(b, b), fmaxf(dot3(c, c), dot3(d, d))));
+  }
+  for (int o = 16; o > 0; o >>= 1) l2 = fmaxf(l2, __shfl_xor_sync(0xffffffffu, l2, o));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = l2;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (float x : part) l2 = fmaxf(l2, x);
+  atomicMax(reinterpret_cast<int*>(&ms->eta), __float_as_int(1e-6f * sqrtf(l2)));   // not negative: ordered as its bits
+}
+
 // The records, bottom-up in one launch: the threads of nodes without internal children start, and the last child
 // to finish takes its parent (done: zeroed counters).
 __global__ void k_hz_nodes(const float4* __restrict__ nodes, const float4* __restrict__ tri, const int* parent, int n4,

@@ -13,12 +13,11 @@ namespace st {
 
 // Mesh facts the primary-visibility bins use to drop back faces: six times the
 // signed volume (its sign tells outward from inward winding) and the vertex
-// bounds as order-preserving ints; and for the horizons the longest edge.
+// bounds as order-preserving ints; and for the free directions, set by their build, the longest edge.
 struct MeshStat {
   double vol6;
   int lo[3], hi[3];
   int winding;   // +1 outward, -1 inward, 0 when the volume is too small against the bounds to tell
-  int lmax2;     // longest edge, squared (float bits)
   float eta;     // 1e-6 of the longest edge: how far beside a triangle the watertight test may report a hit
 };
 

@@ -27,7 +27,7 @@ def _step(scene, sc, w):
     dV, dF = scene.backward(sc.views, B, SEED, w, _opts())
     built = scene.stats()["kernel_launches"]
     scene.backward(sc.views, B, SEED, w, _opts())
-    assert built - scene.stats()["kernel_launches"] == 6 + 2   # primary lists and free directions were built, and then kept
+    assert built - scene.stats()["kernel_launches"] == 6 + 3   # primary lists and free directions were built, and then kept
     sig = torch.zeros(sc.n_pixels, dtype=torch.int64, device="cuda")
     img = scene.render(sc.views, B, SEED, signatures=sig)
     s = scene.stats()
