@@ -68,6 +68,8 @@ constexpr int EDGE_RECORDS = 1 << 15;
 constexpr long long EDGE_RECORD_BYTES = 256LL << 20;
 // Faces per bin cell a view may hold, over the whole screen, before its cells are split further
 constexpr double BIN_FACES_PER_CELL = 0.5;
+// Primary rays, and faces times views, from which a closed mesh's call below a million rays builds lists (plan_call)
+constexpr long long BIN_MIN_RAYS = 5LL << 17, BIN_MIN_LEAVES = 512;
 // Whether a call uses the faces' free directions (uses_free_directions). A face costs 8 (smooth) to 17 ns (rough) to build; a
 // path that hits the mesh wins back what the rays they answer would have cost, which depends on the share of the directions
 // that is free (hz_survey). Hits a face (expected_hits) at which iterations with and without them took the same time,
@@ -858,6 +860,20 @@ st_status enqueue_call(st_scene* s, const Plan& p, int Q, cudaStream_t st, bool 
   return body;
 }
 
+// Faces a warp of k_bin takes: 32, or fewer (a power of two) where that leaves the SMs short of warps. A warp takes its faces
+// with many cells one after the other, so a coarse mesh in few views kept ten warps busy for as long as 32 faces take: an
+// iteration of one view of 320 faces and 655k rays 1842 us, now 555 (617 without lists).
+int bin_faces_per_warp(const st_scene* s, int views) {
+  const long long warps = 16LL * std::max(s->sm_count, 1);
+  int per = 32;
+  while (per > 1 && (long long)s->nf * views < warps * per) per /= 2;
+  return per;
+}
+dim3 bin_grid(const st_scene* s, int views, int per_warp) {
+  const int warps = (s->nf + per_warp - 1) / per_warp, in_block = BIN_BLOCK / 32;
+  return dim3((warps + in_block - 1) / in_block, (unsigned)views);
+}
+
 st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStream_t st, bool host_sized,
                        bool timing) {
   ST_CUDA(cudaMemsetAsync(s->eng.stat, 0, sizeof(unsigned long long) * STAT_SIZE, st));
@@ -889,15 +905,16 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
     long long P = p.cells;
     int nv = (int)p.views.size();
     long long nb = (P + 4095) / 4096;
-    dim3 g((s->nf + 127) / 128, (unsigned)nv);
+    const int per_warp = bin_faces_per_warp(s, nv);
+    const dim3 g = bin_grid(s, nv, per_warp);
     ST_CUDA(cudaMemsetAsync(s->bin_cur, 0, sizeof(int) * P, st));
     k_fill_int<<<(nv + 127) / 128, 128, 0, st>>>(s->bin_ok, nv, 1);
-    k_bin<0><<<g, 128, 0, st>>>(c, nv, s->bin_ok);
+    k_bin<0><<<g, BIN_BLOCK, 0, st>>>(c, nv, s->bin_ok, per_warp);
     k_scan_blocks<<<(unsigned)nb, SCAN_BLOCK, 0, st>>>(s->bin_cur, s->bin_start, P, s->bin_part);
     k_scan_parts<<<1, SCAN_BLOCK, 0, st>>>(s->bin_part, (int)nb, s->bin_start, P);
     k_scan_add<<<(unsigned)nb, SCAN_BLOCK, 0, st>>>(s->bin_start, P, s->bin_part);
     ST_CUDA(cudaMemsetAsync(s->bin_cur, 0, sizeof(int) * P, st));
-    k_bin<1><<<g, 128, 0, st>>>(c, nv, s->bin_ok);
+    k_bin<1><<<g, BIN_BLOCK, 0, st>>>(c, nv, s->bin_ok, per_warp);
     ST_CUDA(copy_async(s->bin_total_host, s->bin_start + P, sizeof(int), cudaMemcpyDeviceToHost, st));
     s->launches += 6;
   }
@@ -911,17 +928,18 @@ st_status enqueue_body(st_scene* s, const Plan& p, const KCtx& c, int Q, cudaStr
     cl.views = s->d_lviews;
     cl.bin_start = s->lbin_start; cl.bin_list = s->lbin_list; cl.bin_cur = s->lbin_cur; cl.bin_ok = s->lbin_ok;
     cl.bin_cap = s->lbin_cap; cl.bin_cells = P;
-    dim3 g((s->nf + 127) / 128, (unsigned)nl);
+    const int per_warp = bin_faces_per_warp(s, nl);
+    const dim3 g = bin_grid(s, nl, per_warp);
     k_fill_int<<<(nl + 127) / 128, 128, 0, st>>>(s->lbin_ok, nl, 1);
     k_light_views<<<nl, LVIEW_BLOCK, 0, st>>>(s->lights, s->verts, s->nv, s->mstat, s->lbin_res, s->d_lviews,
                                              s->lbin_ok);
     ST_CUDA(cudaMemsetAsync(s->lbin_cur, 0, sizeof(int) * P, st));
-    k_bin<0><<<g, 128, 0, st>>>(cl, nl, s->lbin_ok);
+    k_bin<0><<<g, BIN_BLOCK, 0, st>>>(cl, nl, s->lbin_ok, per_warp);
     k_scan_blocks<<<(unsigned)nb, SCAN_BLOCK, 0, st>>>(s->lbin_cur, s->lbin_start, P, s->lbin_part);
     k_scan_parts<<<1, SCAN_BLOCK, 0, st>>>(s->lbin_part, (int)nb, s->lbin_start, P);
     k_scan_add<<<(unsigned)nb, SCAN_BLOCK, 0, st>>>(s->lbin_start, P, s->lbin_part);
     ST_CUDA(cudaMemsetAsync(s->lbin_cur, 0, sizeof(int) * P, st));
-    k_bin<1><<<g, 128, 0, st>>>(cl, nl, s->lbin_ok);
+    k_bin<1><<<g, BIN_BLOCK, 0, st>>>(cl, nl, s->lbin_ok, per_warp);
     ST_CUDA(copy_async(s->lbin_total_host, s->lbin_start + P, sizeof(int), cudaMemcpyDeviceToHost, st));
     s->launches += 7;
   }
@@ -1113,12 +1131,16 @@ st_status plan_call(st_scene* s, const st_view* views, int n_views, int default_
     return fail(ST_ERR_INVALID_ARG, "no light: the scene has none and no view brings one");
   // The lists cost a fixed 30 us (seven launches) and 0.14 ns per face and view to build. Below about a million primary
   // rays that exceeds what they save on an open mesh (three planes, 786k paths: 0.88 ms without, 0.93 with them); on a
-  // closed one they pay from 5 * 2^17 on while there are few faces and views for the rays (MATERIAL). Such calls keep
-  // the back faces in them: at a silhouette edge a ray can hit both faces within rounding, and the tree these calls
-  // used before takes the nearer of the two.
+  // closed one they pay from BIN_MIN_RAYS on while there are few faces and views for the rays, and not next to none.
+  // Iterations of 655k rays, speed with them over without, by faces x views: 20 x 1 0.51, 20 x 16 0.97, 320 x 1 1.11,
+  // 320 x 4 1.25, 1280 x 1 1.23, 1280 x 16 1.44, 5120 x 4 1.46, 6400 x 1 (knot) 1.12, 6400 x 16 1.17 to 1.23, 20480 x 1 1.38,
+  // 20480 x 4 1.49; renders alone 0.31, 0.91, 0.98, 1.24, 1.22, 1.40, 1.41, 1.06, 1.05 to 1.18, 1.18, 1.24. 2^19 rays are within
+  // 0.1 of these (renders of 20480 x 16 lose, 0.98, where 655k win, 1.17). Such calls keep the back faces in them: at a
+  // silhouette edge a ray can hit both faces within rounding, and the tree these calls used before takes the nearer of the two.
   p.cull = s->closed && p.total >= (1LL << 20);
   p.bins = p.total >= (1LL << 20) ||
-           (s->closed && p.total >= (5LL << 17) && (long long)s->nf * n_views <= p.total / 4);
+           (s->closed && p.total >= BIN_MIN_RAYS && (long long)s->nf * n_views >= BIN_MIN_LEAVES &&
+            (long long)s->nf * n_views <= p.total / 4);
   p.lbins = p.total >= (1LL << 20) && s->nl > 0;   // the same limit: the build is a few launches over the faces
   {
     std::vector<std::pair<long long, long long>> rg;

@@ -539,10 +539,11 @@ __device__ __forceinline__ bool hidden_back_face(const KCtx& c, const DevView& v
 // few; a larger box is taken by the whole warp, a cell per lane: a coarse mesh seen at high resolution has hundreds of
 // cells per face, and their atomics one after the other held the launch up (1280 faces, two views of 66 x 433 pixels:
 // 0.60 ms to fill, now 0.03).
-constexpr int BIN_OWN_CELLS = 12;
+constexpr int BIN_OWN_CELLS = 12, BIN_BLOCK = 128;
 template <int FILL>
-__global__ void k_bin(KCtx c, int n_views, int* ok) {
-  const int li = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(BIN_BLOCK) k_bin(KCtx c, int n_views, int* ok, int per_warp) {
+  const int lane = threadIdx.x & 31, warp = (blockIdx.x * BIN_BLOCK + threadIdx.x) >> 5;
+  const int li = lane < per_warp ? warp * per_warp + lane : c.nf;
   const int vi = blockIdx.y;
   if (vi >= n_views) return;
   const DevView v = c.views[vi];
