@@ -445,11 +445,16 @@ struct ScreenTri {
   bool degenerate;
 };
 
+// The lists are counted by one kernel and filled by another, which have to agree on every leaf and cell: one entry more
+// than counted pushes a leaf out of its list, one less leaves an old entry in it. So what decides (the box, the cell test, the
+// back faces) is rounded as written, like shading's sums (st_device.cuh); left to the compiler the two disagreed on a few
+// cells of the 1M-face mesh.
+
 // bin-cell coordinates of a point at rel = X - eye and depth z along fwd (cells: pixels times v.kb)
 __device__ __forceinline__ float2 cell_xy(const DevView& v, float3 rel, float z) {
   const float zz = fmaxf(z, Z_NEAR);
-  return make_float2((dot3(rel, v.right) / (zz * v.kx) + 1.0f) * (float)(v.W * v.kb) * 0.5f,
-                     (1.0f - dot3(rel, v.up) / (zz * v.ky)) * (float)(v.H * v.kb) * 0.5f);
+  return make_float2(__fmul_rn(__fadd_rn(dot_rn(rel, v.right) / __fmul_rn(zz, v.kx), 1.0f), (float)(v.W * v.kb) * 0.5f),
+                     __fmul_rn(__fsub_rn(1.0f, dot_rn(rel, v.up) / __fmul_rn(zz, v.ky)), (float)(v.H * v.kb) * 0.5f));
 }
 
 // 0: cannot be hit from the eye or off screen; 1: box in (x0..x1, y0..y1);
@@ -464,7 +469,7 @@ __device__ __forceinline__ int leaf_screen_box(const DevView& v, float4 a, float
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     float3 rel = P[k] - v.eye;
-    float z = dot3(rel, v.fwd);
+    float z = dot_rn(rel, v.fwd);
     front += z > Z_NEAR;
     behind += z <= 0.0f;
     float2 q = cell_xy(v, rel, z);
@@ -479,16 +484,17 @@ __device__ __forceinline__ int leaf_screen_box(const DevView& v, float4 a, float
   x0 = max(0, (int)floorf(lx)); y0 = max(0, (int)floorf(ly));
   x1 = min(Wc - 1, (int)floorf(hx)); y1 = min(Hc - 1, (int)floorf(hy));
   if ((long long)(x1 - x0 + 1) * (y1 - y0 + 1) > BIN_MAX_BOX) return -1;
-  float area = (px[1] - px[0]) * (py[2] - py[0]) - (py[1] - py[0]) * (px[2] - px[0]);
+  float area = __fmaf_rn(__fsub_rn(px[1], px[0]), __fsub_rn(py[2], py[0]),
+                         -__fmul_rn(__fsub_rn(py[1], py[0]), __fsub_rn(px[2], px[0])));
   et.degenerate = !(fabsf(area) > 1e-6f);
   float sgn = area > 0.0f ? 1.0f : -1.0f;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     int k1 = k == 2 ? 0 : k + 1;
     // E(x, y) = (x - px_k)(py_k1 - py_k) - (y - py_k)(px_k1 - px_k), sign-normalised
-    et.a[k] = -sgn * (py[k1] - py[k]);
-    et.b[k] = sgn * (px[k1] - px[k]);
-    et.c[k] = -(et.a[k] * px[k] + et.b[k] * py[k]);
+    et.a[k] = -sgn * __fsub_rn(py[k1], py[k]);
+    et.b[k] = sgn * __fsub_rn(px[k1], px[k]);
+    et.c[k] = -__fmaf_rn(et.a[k], px[k], __fmul_rn(et.b[k], py[k]));
   }
   return 1;
 }
@@ -500,9 +506,10 @@ __device__ __forceinline__ bool pixel_may_overlap(const ScreenTri& et, int x, in
   for (int k = 0; k < 3; ++k) {
     float cx = et.a[k] > 0.0f ? (float)(x + 1) : (float)x;   // the pixel corner where E is largest
     float cy = et.b[k] > 0.0f ? (float)(y + 1) : (float)y;
-    float e = et.a[k] * cx + et.b[k] * cy + et.c[k];
-    float tol = BIN_PAD * (fabsf(et.a[k]) + fabsf(et.b[k])) + 1e-4f * (fabsf(et.a[k] * cx) + fabsf(et.b[k] * cy) +
-                                                                      fabsf(et.c[k]));
+    const float ax = __fmul_rn(et.a[k], cx), by = __fmul_rn(et.b[k], cy);
+    float e = __fadd_rn(__fadd_rn(ax, by), et.c[k]);
+    float tol = __fmaf_rn(1e-4f, __fadd_rn(__fadd_rn(fabsf(ax), fabsf(by)), fabsf(et.c[k])),
+                          __fmul_rn(BIN_PAD, __fadd_rn(fabsf(et.a[k]), fabsf(et.b[k]))));
     if (e < -tol) return false;
   }
   return true;
@@ -525,13 +532,13 @@ __device__ __forceinline__ bool hidden_back_face(const KCtx& c, const DevView& v
   if (w == 0) return false;
   float3 lo = mk3(from_ordered(c.mstat->lo[0]), from_ordered(c.mstat->lo[1]), from_ordered(c.mstat->lo[2]));
   float3 hi = mk3(from_ordered(c.mstat->hi[0]), from_ordered(c.mstat->hi[1]), from_ordered(c.mstat->hi[2]));
-  float m = 1e-4f * fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z)) + 1e-6f;
+  float m = __fmaf_rn(1e-4f, fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z)), 1e-6f);
   bool outside = v.eye.x < lo.x - m || v.eye.x > hi.x + m || v.eye.y < lo.y - m || v.eye.y > hi.y + m ||
                  v.eye.z < lo.z - m || v.eye.z > hi.z + m;
   if (!outside) return false;
-  float3 n = cross3(xyz(b) - xyz(a), xyz(cc) - xyz(a));
+  float3 n = cross_rn(xyz(b) - xyz(a), xyz(cc) - xyz(a));
   float3 e = v.eye - xyz(a);
-  float f = dot3(n, e), tol = 1e-5f * len3(n) * len3(e);
+  float f = dot_rn(n, e), tol = 1e-5f * sqrtf(dot_rn(n, n)) * sqrtf(dot_rn(e, e));
   return w > 0 ? f < -tol : f > tol;
 }
 
@@ -1043,10 +1050,11 @@ constexpr float SH_NONE = 0.0f, SH_TRACE = 1.0f, SH_FREE = 2.0f;
 // A vertex whose NEE rays all leave above its face's horizon (st_horizon.cuh) adds them here, and a continuation
 // above it escapes here: such a path needs no queue, no ray state and no traversal. The sums take the same terms in
 // the same order as the queued way (k_shadow's lights, then the escape), rounded alike. HZ = false: no free directions
-// are built, every ray is traced (87 registers against 116).
+// are built, every ray is traced.
 // Waits on loads with few warps (a third of the issue slots used at two blocks of 256 per SM), so it is held to seven
-// (without free directions six) blocks of 128: an iteration on 200k faces and 64 views 34.3 -> 31.9 ms, on 5120 faces
-// 3.91 -> 3.63, three planes 0.886 either way. What both variants decide by and add to a pixel is rounded as written.
+// (without free directions six) blocks of 128, 72 and 76 registers, the former with 176 bytes spilled: an iteration on 200k
+// faces and 64 views 34.3 -> 31.9 ms, on 5120 faces 3.91 -> 3.63, three planes 0.886 either way. What both variants decide
+// by and add to a pixel is rounded as written.
 constexpr int SHADE_BLOCK = 128;
 template <bool HZ>
 __global__ void __launch_bounds__(SHADE_BLOCK, HZ ? 7 : 6) k_shade(KCtx c, int b, int first) {
