@@ -23,6 +23,7 @@
 //    largest at the triangle's vertices. m runs over f's edge normals and their
 //    bisectors at f's vertices, which bounds faces that share an edge or a vertex
 //    with f by their slope.
+//    Needles (HZ_THIN) take the sphere instead.
 // k_horizon gives every face a warp, whose lanes take the children of eight nodes
 // at a time: those of f's ancestors, nearest first, then what they open. A node
 // whose cells are all marked already, or that is below f's plane, is dropped; one
@@ -45,9 +46,9 @@
 // origin, and of 10^10 rays past one neighbour, coordinates up to 10^4 and faces from
 // 10^-3 to 5, with and without fused products, no free one hit.)
 //
-// Measured on one GB300. k_horizon is bounded by instruction issue (55 % active, 16 to
-// 24 warps per SM, 15 of 32 lanes: nodes and triangles of a round take different
-// loads): 1.6 ms at 200k smooth faces (12 rounds a face), 0.8 ms at the 50k-face torus
+// Measured on one GB300. k_horizon is bounded by instruction issue (70 % active, 23
+// warps per SM, 15 of 32 lanes at 200k faces: nodes and triangles of a round take
+// different loads): 1.6 ms at 200k smooth faces (12 rounds a face), 0.8 ms at the 50k-face torus
 // knot (24), 16.8 ms at 1M rough ones (25). k_hz_nodes 0.02 to 0.2 ms. Share of the
 // NEE and bounce rays answered: 99 % on the smooth spheres, 53 % on the knot, 80 % on
 // the rough mesh. Of an iteration on 200k faces and 64 views, k_extend and k_shadow
