@@ -44,7 +44,10 @@
 // (Of 6 10^8 sampled free rays, half from within 10^-5 of an edge's length of it, one
 // had such a hit without this. With it: none of 3.4 10^9 over twelve meshes about the
 // origin, and of 10^10 rays past one neighbour, coordinates up to 10^4 and faces from
-// 10^-3 to 5, with and without fused products, no free one hit.)
+// 10^-3 to 5, with and without fused products, no free one hit. 13,700 calls with and
+// without them gave the same images, path signatures and ray counts bitwise, 5,000
+// adjoints the same gradients up to the atomics' order: spheres, fractal ones, torus
+// knots and planes, moved up to 700, scaled from 0.01 to 3, refitted and rebuilt.)
 //
 // Measured on one GB300. k_horizon is bounded by instruction issue (70 % active, 23
 // warps per SM, 15 of 32 lanes at 200k faces: nodes and triangles of a round take
