@@ -78,18 +78,20 @@ constexpr long long BIN_MIN_RAYS = 5LL << 17, BIN_MIN_LEAVES = 512;
 //   0.90 to 0.96 (fractal spheres)               30 to 34 (75)
 //   0.41 to 0.46 (torus knots of 12k to 160k)    50 to 100; listed lights alone 120 to 240; traced lights 30 to 50
 //   0.23 to 0.33 (rougher spheres, any size)     none up to 1500 (0.90 to 0.99 of the speed without)
-//   0.28 to 0.33 (three planes, open)            below 270 (1.04 to 1.2 from there on)
+//   0.28 to 0.33 (three planes seen from inside) none up to 500 (listed lights alone 0.89 to 0.93); traced lights below 45
+//   1.00 (the planes' outer sides, open)         60; traced lights below 45
 // Rays to the scene's listed lights (see light_bin_range) cost little without, and bounces after the first count for
 // little, since few paths get there: a call of listed lights and one vertex a path loses on any but smooth meshes (0.98 at
-// 280). A build that serves a forward call alone takes half as much again, on concave meshes twice. Below HZ_MIN_JOBS paths
-// the two launches' latency (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN: three planes of 384 and 6144
-// faces 0.97 and 0.94 at 786k paths, 1.04 and 1.01 at 2^20 (renders 1.05, 0.98), 1.04 at 2^21 (1.04, 1.02). An open sphere
+// 280). A build that serves a forward call alone takes half as much again, on closed concave meshes twice. Below HZ_MIN_JOBS paths
+// the two launches' latency (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN: the outer sides of three
+// planes of 384 and 6144 faces 0.97 and 0.94 at 786k paths, 1.04 and 1.01 at 2^20 (renders 1.05, 0.98), 1.04 at 2^21 (1.04, 1.02). An open sphere
 // would win from 2^19 on (1.09, at 2^20 1.39; a render 0.99, 1.35).
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
 constexpr double HZ_SMOOTH = 0.95, HZ_FRACTAL = 0.7, HZ_CONCAVE = 0.35;   // least shares of free directions
 constexpr int HZ_HITS_SMOOTH = 13, HZ_HITS_FRACTAL = 35, HZ_HITS_CONCAVE = 52, HZ_HITS_CONCAVE_LISTED = 160,
-              HZ_HITS_CONCAVE_TRACED = 44, HZ_HITS_OPEN = 230;
+              HZ_HITS_CONCAVE_TRACED = 44;
 constexpr double HZ_ALONE = 1.5, HZ_ALONE_CONCAVE = 2.0;
+constexpr double HZ_OPEN = 4.0;   // an open mesh is seen from both sides, and one of them has no directions
 // Longest edge from which no direction is usable: the directions' margins grow with it (by a tenth of its length in the sine
 // of elevation, T_EPS being fixed). What a smooth sphere of 20k faces and 256 rays a face won, 0.48 ms of the 1.26 an
 // iteration takes at a longest edge of 0.05, was 0.33 at 1, 0.14 at 3, 0.06 at 5 and nothing at 8.5 (the build takes
@@ -1186,10 +1188,11 @@ bool uses_free_directions(const st_scene* s, const Plan& p) {
   const bool env = s->env.w > 0, traced = p.max_vl > 0 || (s->nl > 0 && !p.lbins), smooth = s->hz_free >= HZ_SMOOTH,
              fractal = s->hz_free >= HZ_FRACTAL, built = s->hz_valid && s->hz_geom == s->geom_version;
   if (built && fractal) return true;   // as the call that built them decided
-  if (s->closed && s->hz_free < HZ_CONCAVE) return false;
+  if (s->hz_free < HZ_CONCAVE && (s->closed || !traced)) return false;
   if (p.B == 1 && !env && !traced && !smooth) return false;
-  double need = smooth ? HZ_HITS_SMOOTH : fractal ? HZ_HITS_FRACTAL : !s->closed ? HZ_HITS_OPEN : traced ? HZ_HITS_CONCAVE_TRACED
+  double need = smooth ? HZ_HITS_SMOOTH : fractal ? HZ_HITS_FRACTAL : traced ? HZ_HITS_CONCAVE_TRACED
               : env ? HZ_HITS_CONCAVE : HZ_HITS_CONCAVE_LISTED;
+  if (!s->closed && !traced) need *= HZ_OPEN;
   if (p.B == 1 && !traced) need *= env ? 2.0 : 8.0;
   double hits = expected_hits(s, p, false);
   if (!built) {   // the mean of the two calls, none for one too small to use them; a call alone asks HZ_ALONE times as much
@@ -1197,7 +1200,7 @@ bool uses_free_directions(const st_scene* s, const Plan& p) {
     for (const Seg& sg : p.segs) camera += sg.kind == 0 ? sg.count : 0;
     if (p.kind == 1) hits = 0.5 * (hits + (camera >= least ? expected_hits(s, p, true) : 0.0));
     else if (s->adj_seen && s->geom_version - s->adj_geom <= 1) hits = 0.5 * (hits + s->adj_hits);
-    else need *= fractal ? HZ_ALONE : HZ_ALONE_CONCAVE;
+    else need *= fractal || !s->closed ? HZ_ALONE : HZ_ALONE_CONCAVE;
   }
   return hits * s->hz_reach * s->hz_reach >= need * s->nf;
 }

@@ -102,3 +102,31 @@ def test_paths_that_miss_do_not_count(st):  # noqa: F811
     """As many paths in wide views, most of which look past the mesh."""
     assert _builds(st, "smooth", "env", 3, 1.0, True)
     assert not _builds(st, "smooth", "env", 3, 1.0, True, w=512, h=32)
+
+
+@pytest.mark.parametrize("side,light,n,adjoint,builds", [
+    ("outer", "env", 48, True, True), ("outer", "env", 48, False, True), ("outer", "env", 64, False, False),
+    ("outer", "env", 72, True, False), ("inner", "env", 8, True, False), ("inner", "view", 32, True, True),
+    ("inner", "view", 80, True, False)])
+def test_open_meshes(st, side, light, n, adjoint, builds):  # noqa: F811
+    """Three planes of n x n quads each, 6 n^2 faces, from 2^21 paths on: the side that has directions is the one outward of
+    the origin, where the planes see nothing (52 hits a face, alone 78) or one another (no build without traced lights)."""
+    sc = S.color_bleed(n=n)
+    rng = np.random.default_rng(2)
+    views = S.fibonacci_views(4, [256] * 4, [256] * 4, [9] * 4)   # about 1.3 million hits
+    if light == "view":
+        views = S.with_view_lights(views)
+    sc = S.Scene("open", S._f32(sc.vertices - (0.5 if side == "outer" else 0.0)), sc.faces, sc.face_params,
+                 env=S.lognormal_env(rng, 64, 32) if light == "env" else None, views=views, max_bounces=3)
+    assert sum(v.width * v.height * v.spp for v in views) >= 1 << 21
+    scene = st.Scene.from_scene(sc)
+    counts = []
+    for _ in range(2):
+        if adjoint:
+            scene.backward(views, 3, 1, torch.ones((sc.n_pixels, 3), device="cuda"), st.make_opts(edge_term=0))
+        else:
+            scene.render(views, 3, 1)
+        counts.append(scene.stats()["kernel_launches"])
+        assert scene.stats()["device_error"] == 0
+    scene.close()
+    assert counts[0] - counts[1] == 6 + (3 if builds else 0)   # the primary lists, and the free directions
