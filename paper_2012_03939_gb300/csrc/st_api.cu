@@ -82,10 +82,11 @@ constexpr long long BIN_MIN_RAYS = 5LL << 17, BIN_MIN_LEAVES = 512;
 //   1.00 (the planes' outer sides, open)         60; traced lights below 45
 // Rays to the scene's listed lights (see light_bin_range) cost little without, and bounces after the first count for
 // little, since few paths get there: a call of listed lights and one vertex a path loses on any but smooth meshes (0.98 at
-// 280). A build that serves a forward call alone takes half as much again, on closed concave meshes twice. Below HZ_MIN_JOBS paths
-// the two launches' latency (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN: the outer sides of three
-// planes of 384 and 6144 faces 0.97 and 0.94 at 786k paths, 1.04 and 1.01 at 2^20 (renders 1.05, 0.98), 1.04 at 2^21 (1.04, 1.02). An open sphere
-// would win from 2^19 on (1.09, at 2^20 1.39; a render 0.99, 1.35).
+// 280). A build that serves a forward call alone takes half as much again, on closed concave meshes twice. Below
+// HZ_MIN_JOBS paths the two launches' latency (50 us) is not won back; on an open mesh not below HZ_MIN_JOBS_OPEN: the outer
+// sides of three planes of 384 and 6144 faces 0.97 and 0.94 at 786k paths, 1.04 and 1.01 at 2^20 (renders 1.05, 0.98), 1.04
+// at 2^21 (1.04, 1.02). An open sphere would win from 2^19 on (1.09, at 2^20 1.39; a render 0.99, 1.35). Not built, the
+// inside of 2166 faces of planes under two listed lights, 30 views of 435 x 70, takes 5.72 ms an iteration; built, 6.23.
 constexpr long long HZ_MIN_JOBS = 1LL << 19, HZ_MIN_JOBS_OPEN = 1LL << 21;
 constexpr double HZ_SMOOTH = 0.95, HZ_FRACTAL = 0.7, HZ_CONCAVE = 0.35;   // least shares of free directions
 constexpr int HZ_HITS_SMOOTH = 13, HZ_HITS_FRACTAL = 35, HZ_HITS_CONCAVE = 52, HZ_HITS_CONCAVE_LISTED = 160,
